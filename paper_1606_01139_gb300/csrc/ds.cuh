@@ -47,6 +47,25 @@ __device__ __forceinline__ void split_bits(double x, float& hi, float& lo) {
   }
 }
 
+// The same split without an FP64 instruction on any path (GB300's FP64 pipe
+// would be held by every warp with one lane on it): magnitudes below 2^-74 go
+// to (0, 0) and the exponent is capped at 2^126, for operands known to lie far
+// inside that range (unit vectors, projected matrices, their coefficients).
+__device__ __forceinline__ void split_flush(double x, float& hi, float& lo) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const unsigned int top = (unsigned int)(b >> 32);
+  const unsigned int sgn = top & 0x80000000u;
+  const int e0 = (int)((top >> 20) & 0x7ff);
+  const bool small = e0 < 949;
+  const int e = min(max(e0, 949), 1149);
+  const unsigned int up = (unsigned int)(b >> 28) & 1u;
+  const unsigned int fb = ((unsigned int)(e - 896) << 23 | ((unsigned int)(b >> 29) & 0x7fffffu)) + up;
+  const int rem = (int)((unsigned int)b & 0x1fffffffu) - (int)(up << 29);
+  const float t = (float)rem * __uint_as_float((unsigned int)(e - 948) << 23);
+  hi = small ? 0.f : __uint_as_float(sgn | fb);
+  lo = small ? 0.f : (sgn ? -t : t);
+}
+
 // (s, e) += a * b with a, b double-single: the product is formed exactly up to
 // its tail with FMA, the head added with TwoSum (Knuth), errors kept in e.
 __device__ __forceinline__ void fma_acc(float& s, float& e, float ah, float al, float bh, float bl) {

@@ -46,6 +46,9 @@ struct SV {
   using Sig = std::conditional_t<DS, double, float>;
 };
 
+// forms of the projected Schur step, in the order they are tried
+enum { kFormMp = 0, kFormDs = 1, kFormF64 = 2 };
+
 template <bool DS>
 struct SvWin {
   using T = typename SV<DS>::T;
@@ -54,8 +57,9 @@ struct SvWin {
   int nreq = 0, m = 0, keep = 0, ldq = 0, ldh = 0, col = 0;
   int p = 0;  // the newest block is basis columns [p, p + nb) (the ones expanded next)
   DevMem Q, H, Z, S, Bz, theta, resid, Yw, eps_w, res_w, Hw, Zw, C1, C2, Z32, rinv, part;  // part: FP64 chunk partials
-  DevMem Hsave;          // the projected matrix of the Schur step in flight (for a retry in FP64)
-  bool retry = false;    // the double-single step gave up; the FP64 step runs on the saved matrix
+  DevMem Hsave;          // the projected matrix of the Schur step in flight (for a retry)
+  DevMem mpw;            // work of the restart's form of the step (schur_mp.cu)
+  int form = 0;          // kernel of the Schur step in flight: kFormMp, kFormDs or kFormF64
   int schur_retries = 0;
   bool done = false, failed = false;
   long long matvecs = 0;
@@ -180,6 +184,7 @@ swi_status solve_sv(swi_ctx* c, const swi_solve_opts& opt, swi_solve_info* info)
     w.Hw.ensure(16 * hh);
     w.Zw.ensure(16 * hh);
     w.Hsave.ensure(sizeof(double2) * hh);
+    if (w.m <= swi::kMpMaxOrder) w.mpw.ensure(swi::mp_schur_bytes(w.m, w.m - nb, w.ldh, nb));
     w.Yw.ensure(sizeof(double2) * w.ldh * w.nreq);
     w.eps_w.ensure(sizeof(double2) * w.nreq);
     w.res_w.ensure(sizeof(double) * w.nreq);
@@ -341,14 +346,15 @@ swi_status solve_sv(swi_ctx* c, const swi_solve_opts& opt, swi_solve_info* info)
     }
   };
 
-  // the projected eigenproblem of window j (order w.p) on its own stream; the
-  // double-single kernel, or after it gave up the native FP64 one on the
-  // saved matrix
-  auto launch_schur = [&](Win& w, bool f64) {
+  // the projected eigenproblem of window j (order w.p) on its own stream: the
+  // restart's form (schur_mp.cu) where the order allows it, after it gave up
+  // the double-single kernel, and after that the native FP64 one, on the saved
+  // matrix
+  auto launch_schur = [&](Win& w, int form) {
     const int j = w.col;
     cudaStream_t sj = side.st[j];
     const size_t hh = (size_t)w.ldh * w.ldh;
-    if (f64) SWI_CUDA_TRY(cudaMemcpyAsync(w.H.p, w.Hsave.p, sizeof(double2) * hh, cudaMemcpyDeviceToDevice, sj));
+    if (form > w.form) SWI_CUDA_TRY(cudaMemcpyAsync(w.H.p, w.Hsave.p, sizeof(double2) * hh, cudaMemcpyDeviceToDevice, sj));
     else SWI_CUDA_TRY(cudaMemcpyAsync(w.Hsave.p, w.H.p, sizeof(double2) * hh, cudaMemcpyDeviceToDevice, sj));
     // as ARPACK does, keep more Ritz vectors once some wanted pairs have converged
     const int keep_eff = std::min(w.m - nb, w.keep + std::min(w.nconv, (w.m - w.keep) / 2));
@@ -360,10 +366,14 @@ swi_status solve_sv(swi_ctx* c, const swi_solve_opts& opt, swi_solve_info* info)
                               w.theta.template as<double2>(), w.resid.template as<double>(), w.S.template as<double2>(),
                               c->ordinfo.as<int>() + 4 * j, w.p, w.ldh, nb, keep_eff, w.nreq, w.m - nb, tol_abs,
                               w.Hw.p, w.Zw.p, w.sig_im};
+    if (form == kFormMp && !(w.p <= w.m && w.mpw.p && swi::mp_schur_takes(w.p, keep_eff, w.m - nb))) form = kFormDs;
+    w.form = form;
     {
       ProfScope ps(c, SWI_K_SCHUR, 0.0, 0.0, sj);
-      if (f64) swi::launch_schur_batch(sb, sj, &c->launches);
-      else swi::launch_schur_ds_batch(sb, sj, &c->launches);
+      if (form == kFormMp)
+        swi::launch_schur_mp(sb.job[0], w.mpw.p, std::min(keep_eff + 8, w.m - nb), sj, &c->launches);
+      else if (form == kFormDs) swi::launch_schur_ds_batch(sb, sj, &c->launches);
+      else swi::launch_schur_batch(sb, sj, &c->launches);
     }
     SWI_CUDA_TRY(cudaMemcpyAsync(side.oi + 4 * j, c->ordinfo.as<int>() + 4 * j, sizeof(int) * 4,
                                  cudaMemcpyDeviceToHost, sj));
@@ -376,17 +386,17 @@ swi_status solve_sv(swi_ctx* c, const swi_solve_opts& opt, swi_solve_info* info)
     const int* oi = side.oi + 4 * j;
     const int kk = oi[0], nconv = oi[1], st = oi[2];
     const int n = w.p;  // order of the projected matrix
-    if (st != 0 && !w.retry) {  // the double-single QR gave up: the FP64 kernel on the same matrix
-      w.retry = true;
-      w.schur_retries++;
-      launch_schur(w, true);
+    if (st != 0 && w.form < kFormF64) {  // it gave up: the next form on the same matrix
+      if (w.form == kFormDs) w.schur_retries++;
+      launch_schur(w, w.form + 1);
       return;
     }
-    w.retry = false;
+    const int order = w.form == kFormMp ? kk : n;  // of the accurate reduction (work accounting)
+    w.form = kFormMp;
     SWI_CUDA_TRY(cudaStreamWaitEvent(c->stream, side.done[j], 0));
     w.restarts++;
     w.nconv = nconv;
-    if (c->prof_on) c->schur_flops += 64.0 / 3.0 * (double)n * n * n + 20.0 * 1024.0 * (double)oi[3];
+    if (c->prof_on) c->schur_flops += 64.0 / 3.0 * (double)order * order * order + 20.0 * 1024.0 * (double)oi[3];
     if (st != 0) w.failed = true;
     if (st != 0 || nconv >= w.nreq || w.matvecs >= budget) {
       // Ritz vectors of the wanted pairs into Uall (complex128)
@@ -529,7 +539,7 @@ swi_status solve_sv(swi_ctx* c, const swi_solve_opts& opt, swi_solve_info* info)
       if (w.p + nb <= w.m) continue;
       SWI_CUDA_TRY(cudaEventRecord(side.ready[j], c->stream));
       SWI_CUDA_TRY(cudaStreamWaitEvent(side.st[j], side.ready[j], 0));
-      launch_schur(w, false);
+      launch_schur(w, kFormMp);
     }
     SWI_CUDA_TRY(cudaEventRecord(side.lag[step & 1], c->stream));
   }

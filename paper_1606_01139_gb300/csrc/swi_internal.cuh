@@ -76,6 +76,11 @@ struct Error {
 
 #define SWI_CHECK_LAUNCH() SWI_CUDA_TRY(cudaGetLastError())
 
+// Lets a kernel use all the shared memory a block may have beside its static
+// share, once per kernel and device.  (Setting the size of each launch instead
+// races between host threads: one lowers the limit under another's launch.)
+void smem_opt_in(const void* kernel);
+
 // ---------------------------------------------------------------- operator data
 struct StencilParams {
   int nx, ny, nz;
@@ -210,6 +215,33 @@ struct SchurBatch {
 void launch_schur_batch(const SchurBatch& b, cudaStream_t s, long long* launches);
 // The same step in double-single arithmetic (schur_ds.cu); needs Hw, Zw.
 void launch_schur_ds_batch(const SchurBatch& b, cudaStream_t s, long long* launches);
+
+// The restart's form of the step (schur_mp.cu): the kept block alone to
+// double-single accuracy, from an FP32 Schur form.  On exit H[0:k, 0:k] = T_kk,
+// Z[:, 0:k], Bz, theta, resid, S and ordinfo as above (the rest of H and Z is
+// not written); ordinfo[2] != 0 when it gave up (H then needs its saved copy).
+constexpr int kMpMaxOrder = 512;
+struct MpJob {
+  int m, ld, b, keep, kmax, kcap, nwant, max_steps, max_steps2, max_stepsk;
+  double sig_im, tol_abs;
+  double2* H;
+  double2* Z;
+  const double2* B;
+  double2 *Bz, *theta, *S;
+  double* resid;
+  int* ordinfo;
+  int* ctl;                                                // control block (enum CTL_*)
+  float2 *H32, *Hp, *Vr, *Q, *P, *T, *Tr, *R32, *X, *S32;       // FP32 work
+  float* tau;
+  float4 *rot, *rot2, *rotk;                               // rotation lists
+  double2 *V[2], *W, *G, *BV;
+  void *Gd, *Gp, *Vk, *tauk;                               // kept block in double-single
+};
+bool mp_schur_takes(int m, int keep, int kmax);
+// work of launch_schur_mp for orders up to m, kept counts up to kcap
+size_t mp_schur_bytes(int m, int kcap, int ld, int b);
+size_t mp_schur_layout(MpJob* J, void* base, int m, int kcap, int ld, int b);
+void launch_schur_mp(const SchurJob& S, void* work, int kcap, cudaStream_t s, long long* launches);
 
 // Ritz coefficient matrix of the wanted pairs after a Schur step:
 // Yw[:, q] = Z[:, 0:k] s_{w_q} (m x nwant, [m][ld]) and eps_w[q] = theta_{w_q} + sigma,
