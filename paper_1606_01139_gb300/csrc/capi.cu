@@ -108,6 +108,7 @@ swi::StencilParams stencil_params(const swi_ctx* c) {
   for (int m = 0; m < 7; ++m) P.cm[m] = -kFD[m] / (2.0 * c->h * c->h);
   P.V = c->V.as<double>();
   P.G = c->G.as<double>();
+  P.VGds = c->VGds.as<float4>();
   return P;
 }
 
@@ -127,14 +128,17 @@ void sync(cudaStream_t s) { SWI_CUDA_TRY(cudaStreamSynchronize(s)); }
 // Y[:, c] = (A - sigma_c) X[:, c] in chunks of columns, sigma from the context's sigma table
 void apply_block(swi_ctx* c, const double2* X, int ldx, double2* Y, int ldy, int ncols, bool ds) {
   const swi::StencilParams P = stencil_params(c);
+  if (ds) {
+    c->pad_ds.ensure(swi::stencil_ds_work_bytes(P, ncols));
+    swi::launch_stencil_ds(P, X, ldx, Y, ldy, ncols, 0, c->sig_dev.as<double>(), c->pad_ds.as<float4>(), c->stream,
+                           &c->launches);
+    return;
+  }
   for (int c0 = 0; c0 < ncols; c0 += 32) {
     swi::StencilBatch bt;
     bt.n = 1;
     bt.blk[0] = swi::StencilBlock{X + c0, Y + c0, ldx, ldy, std::min(32, ncols - c0), c0};
-    if (ds)
-      swi::launch_stencil_ds(P, bt, c->sig_dev.as<double>(), c->stream, &c->launches);
-    else
-      swi::launch_stencil(P, bt, c->sig_dev.as<double>(), c->stream, &c->launches);
+    swi::launch_stencil(P, bt, c->sig_dev.as<double>(), c->stream, &c->launches);
   }
 }
 
@@ -386,6 +390,8 @@ swi_status do_solve(swi_ctx* c, const swi_solve_opts* o, swi_solve_info* info) {
     if (c->arith != SWI_ARITH_F64) {
       w.Hw.ensure(16 * (size_t)w.ld * w.ld);
       w.Zw.ensure(16 * (size_t)w.ld * w.ld);
+      w.Hsave.ensure(sizeof(double2) * w.ld * w.ld);
+      if (w.m <= swi::kMpMaxOrder) w.mpw.ensure(swi::mp_schur_bytes(w.m, w.m - b, w.ld, b));
     }
     w.Yw.ensure(sizeof(double2) * w.ld * w.nreq);
     w.eps_w.ensure(sizeof(double2) * w.nreq);
@@ -465,15 +471,55 @@ swi_status do_solve(swi_ctx* c, const swi_solve_opts* o, swi_solve_info* info) {
   for (auto& e : side.lag) SWI_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   std::vector<int> in_schur(nwin, 0);
 
+  // The projected eigenproblem of window j (order w.p) on its own stream: the
+  // restart's form (schur_mp.cu) where the order allows it, after it gave up the
+  // double-single kernel on the saved matrix; native FP64 with that arithmetic
+  auto launch_schur = [&](int j, bool again) {
+    Window& w = *win[j];
+    cudaStream_t sj = side.st[j];
+    const size_t hb = sizeof(double2) * (size_t)w.ld * w.ld;
+    // As ARPACK does, keep more Ritz vectors once some wanted pairs have
+    // converged, so the rest keep room in the restarted basis.
+    const int keep_eff = std::min(w.m - b, w.keep + std::min(w.nconv, (w.m - w.keep) / 2));
+    swi::SchurBatch sb;
+    sb.n = 1;
+    sb.job[0] = swi::SchurJob{w.H.as<double2>(), w.Z.as<double2>(), w.Bm.as<double2>(), w.Bz.as<double2>(),
+                              w.theta.as<double2>(), w.resid.as<double>(), w.S.as<double2>(),
+                              c->ordinfo.as<int>() + 4 * j, w.p, w.ld, b, keep_eff, w.nreq, w.m - b, tol_abs,
+                              w.Hw.p, w.Zw.p};
+    w.retried = again;
+    {
+      ProfScope ps(c, SWI_K_SCHUR, 0.0, 0.0, sj);
+      if (c->arith == SWI_ARITH_F64) {
+        swi::launch_schur_batch(sb, sj, &c->launches);
+      } else if (!again && w.mpw.p && swi::mp_schur_takes(w.p, keep_eff, w.m - b)) {
+        SWI_CUDA_TRY(cudaMemcpyAsync(w.Hsave.p, w.H.p, hb, cudaMemcpyDeviceToDevice, sj));
+        swi::launch_schur_mp(sb.job[0], w.mpw.p, std::min(keep_eff + 8, w.m - b), sj, &c->launches);
+      } else {
+        if (again) SWI_CUDA_TRY(cudaMemcpyAsync(w.H.p, w.Hsave.p, hb, cudaMemcpyDeviceToDevice, sj));
+        w.retried = true;
+        swi::launch_schur_ds_batch(sb, sj, &c->launches);
+      }
+    }
+    SWI_CUDA_TRY(cudaMemcpyAsync(side.oi + 4 * j, c->ordinfo.as<int>() + 4 * j, sizeof(int) * 4,
+                                 cudaMemcpyDeviceToHost, sj));
+    SWI_CUDA_TRY(cudaEventRecord(side.done[j], sj));
+    in_schur[j] = 1;
+  };
+
   // Act on a finished Schur step of window j: finalise or thick-restart (context stream).
   auto finish_restart = [&](int j) {
     Window& w = *win[j];
     const int* oi = side.oi + 4 * j;
     const int k = oi[0], nconv = oi[1], st = oi[2];
+    if (st != 0 && c->arith != SWI_ARITH_F64 && !w.retried) {
+      launch_schur(j, true);
+      return;
+    }
     if (c->prof_on && c->arith != SWI_ARITH_F64) {
       // Hessenberg reduction with accumulation ~ 64/3 m^3 real flops, plus 20
       // flops per complex Givens pair update counted by the kernel
-      const double mm = (double)w.p;
+      const double mm = (double)(w.retried ? w.p : k);  // the order of the accurate reduction
       c->schur_flops += 64.0 / 3.0 * mm * mm * mm + 20.0 * 1024.0 * (double)oi[3];
     }
     SWI_CUDA_TRY(cudaStreamWaitEvent(c->stream, side.done[j], 0));
@@ -548,7 +594,7 @@ swi_status do_solve(swi_ctx* c, const swi_solve_opts* o, swi_solve_info* info) {
       continue;
     }
     const int na = (int)act.size();
-    // 1) W_j = (A - sigma_j) V_j for every active window, one launch
+    // 1) W_j = (A - sigma_j) V_j for every active window
     {
       swi::StencilBatch sb;
       sb.n = na;
@@ -559,10 +605,16 @@ swi_status do_solve(swi_ctx* c, const swi_solve_opts* o, swi_solve_info* info) {
       }
       const double Nn = (double)c->N;
       ProfScope ps(c, SWI_K_STENCIL, kStencilFlops * Nn * b * na, (32.0 * b + 16.0) * Nn * na);
-      if (c->arith == SWI_ARITH_F64)
+      if (c->arith == SWI_ARITH_F64) {
         swi::launch_stencil(P, sb, c->sig_dev.as<double>(), c->stream, &c->launches);
-      else
-        swi::launch_stencil_ds(P, sb, c->sig_dev.as<double>(), c->stream, &c->launches);
+      } else {
+        c->pad_ds.ensure(swi::stencil_ds_work_bytes(P, b));
+        for (int q = 0; q < na; ++q) {
+          const swi::StencilBlock& B = sb.blk[q];
+          swi::launch_stencil_ds(P, B.X, B.ldx, B.Y, B.ldy, B.ncols, 0, c->sig_dev.as<double>() + B.sigma_off,
+                                 c->pad_ds.as<float4>(), c->stream, &c->launches);
+        }
+      }
     }
     // 2) block classical Gram-Schmidt, twice, against [Q_j V_j]
     for (int pass = 0; pass < 2; ++pass) {
@@ -617,26 +669,9 @@ swi_status do_solve(swi_ctx* c, const swi_solve_opts* o, swi_solve_info* info) {
       w.matvecs += b;
       if (w.p + b <= w.m) continue;
       if (w.p > w.m || w.keep + b > w.m) throw Error{SWI_ECUDA, "internal: basis bookkeeping out of range"};
-      // As ARPACK does, keep more Ritz vectors once some wanted pairs have
-      // converged, so the rest keep room in the restarted basis.
-      const int keep_eff = std::min(w.m - b, w.keep + std::min(w.nconv, (w.m - w.keep) / 2));
-      swi::SchurBatch sb;
-      sb.n = 1;
-      sb.job[0] = swi::SchurJob{w.H.as<double2>(), w.Z.as<double2>(), w.Bm.as<double2>(), w.Bz.as<double2>(),
-                                w.theta.as<double2>(), w.resid.as<double>(), w.S.as<double2>(),
-                                c->ordinfo.as<int>() + 4 * j, w.p, w.ld, b, keep_eff, w.nreq, w.m - b, tol_abs,
-                                w.Hw.p, w.Zw.p};
       SWI_CUDA_TRY(cudaEventRecord(side.ready[j], c->stream));
       SWI_CUDA_TRY(cudaStreamWaitEvent(side.st[j], side.ready[j], 0));
-      {
-        ProfScope ps(c, SWI_K_SCHUR, 0.0, 0.0, side.st[j]);
-        if (c->arith == SWI_ARITH_F64) swi::launch_schur_batch(sb, side.st[j], &c->launches);
-        else swi::launch_schur_ds_batch(sb, side.st[j], &c->launches);
-      }
-      SWI_CUDA_TRY(cudaMemcpyAsync(side.oi + 4 * j, c->ordinfo.as<int>() + 4 * j, sizeof(int) * 4,
-                                   cudaMemcpyDeviceToHost, side.st[j]));
-      SWI_CUDA_TRY(cudaEventRecord(side.done[j], side.st[j]));
-      in_schur[j] = 1;
+      launch_schur(j, false);
     }
     SWI_CUDA_TRY(cudaEventRecord(side.lag[step & 1], c->stream));
   }
@@ -1081,11 +1116,13 @@ swi_status swi_create(swi_ctx** out, int nx, int ny, int nz, double h, int bc, i
   return SWI_OK;
 }
 
-// the packed (V, Gamma) planes of the TMA-staged complex64 stencil, once both are set
+// the packed (V, Gamma) arrays of the TMA-staged complex64 and the double-single stencils, once both are set
 static void refresh_vg(swi_ctx* c) {
   if (!c->has_V || !c->has_G) return;
   const size_t nxp = (size_t)(c->nx + (c->nx & 1));
   c->VG32.ensure(sizeof(float2) * nxp * c->ny * c->nz);
+  c->VGds.ensure(sizeof(float4) * (size_t)c->N);
+  swi::launch_pack_vg_ds(c->V.as<double>(), c->G.as<double>(), c->N, c->VGds.as<float4>(), c->stream);
   swi::launch_pack_vg(c->V32.as<float>(), c->G32.as<float>(), c->nx, c->ny, c->nz, c->VG32.as<float2>(), c->stream);
   sync(c->stream);
 }

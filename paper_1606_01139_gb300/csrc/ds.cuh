@@ -66,6 +66,37 @@ __device__ __forceinline__ void split_flush(double x, float& hi, float& lo) {
   lo = small ? 0.f : (sgn ? -t : t);
 }
 
+// The same for any magnitude that a float can hold, still without FP64: below
+// 2^-74 the exponent is raised by 64 first and the parts are scaled back (their
+// tails then lie in or below the float denormals); below 2^-138 to (0, 0).
+__device__ __forceinline__ void split_wide(double x, float& hi, float& lo) {
+  unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const bool tiny = ((unsigned int)(b >> 52) & 0x7ffu) < 949u;
+  if (tiny) b += 64ull << 52;
+  const float back = tiny ? 5.421010862427522e-20f : 1.f;  // 2^-64
+  split_flush(__longlong_as_double((long long)b), hi, lo);
+  hi *= back;
+  lo *= back;
+}
+
+// h + l as a double without an FP64 instruction, for a normalised pair (|l| at
+// most half an ulp of h), rounded to nearest: l is rounded to units of the
+// double's last place and added to the mantissa bits.  Magnitudes below 2^-73 or
+// beyond the float range take the FP64 route.
+__device__ __forceinline__ double join_bits(float h, float l) {
+  const unsigned int b = __float_as_uint(h);
+  const unsigned int e = (b >> 23) & 0xffu;
+  if (e >= 54u && e <= 254u) {
+    const unsigned int man = b & 0x7fffffu, top = b & 0x80000000u;
+    const float ls = __uint_as_float(__float_as_uint(l) ^ top);  // l relative to the sign of h
+    const unsigned int below = (man == 0u && ls < 0.f) ? 1u : 0u;  // the next lower binade: half the unit
+    const int k = __float2int_rn(ls * __uint_as_float((306u - e + below) << 23));
+    const long long m = ((long long)((unsigned long long)(e + 896u) << 52 | (unsigned long long)man << 29)) + k;
+    return __longlong_as_double(m | (long long)((unsigned long long)top << 32));
+  }
+  return (double)h + (double)l;
+}
+
 // (s, e) += a * b with a, b double-single: the product is formed exactly up to
 // its tail with FMA, the head added with TwoSum (Knuth), errors kept in e.
 __device__ __forceinline__ void fma_acc(float& s, float& e, float ah, float al, float bh, float bl) {

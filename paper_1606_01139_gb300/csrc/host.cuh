@@ -57,8 +57,9 @@ struct Window {
   double sigma = 0.0;
   int nreq = 0, m = 0, keep = 0, ld = 0;  // ld: columns of the Q buffers (m + b)
   DevMem Q[2], W, H, Bm, Z, S, Bz, theta, resid, C1, C2, G, R1, R1i, R2, R2i, Zext, Yw, eps_w, res_w, Hw, Zw;
+  DevMem mpw, Hsave;  // work of the restart's form of the Schur step, the matrix for a second try
   int cur = 0, p = 0;
-  bool done = false, failed = false;
+  bool done = false, failed = false, retried = false;
   long long matvecs = 0;
   int restarts = 0;
   int nconv = 0;
@@ -78,6 +79,8 @@ struct swi_ctx {
   DevMem V, G, gL, gR;
   DevMem V32, G32;  // FP32 copies for the complex64 stencil
   DevMem VG32;      // (V, Gamma) pairs with even row length, for the TMA-staged stencil
+  DevMem VGds;      // (V, Gamma) split into floats, for the double-single stencil
+  DevMem pad_ds;    // its padded, split copy of the vectors
   bool has_V = false, has_G = false;
   double maxabsV = 0.0, maxG = 0.0;
   std::vector<double> sigma;

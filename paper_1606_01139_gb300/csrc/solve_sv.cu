@@ -221,16 +221,12 @@ swi_status solve_sv(swi_ctx* c, const swi_solve_opts& opt, swi_solve_info* info)
     sync(c->stream);
   }
   const swi::StencilParams P64 = stencil_params(c);
+  if (DS) c->pad_ds.ensure(swi::stencil_ds_work_bytes(P64, ncv));
   const swi::StencilC64Params P32 = stencil_c64_params(c);
   auto apply_all = [&]() {
     if constexpr (DS) {
-      swi::StencilBatch sb;
-      sb.n = 0;
-      for (int c0 = 0; c0 < ncv; c0 += 32)
-        sb.blk[sb.n++] = swi::StencilBlock{reinterpret_cast<const double2*>(Vcur.p) + c0,
-                                           reinterpret_cast<double2*>(Wblk.p) + c0, ldv, ldv,
-                                           std::min(32, ncv - c0), c0, 1};
-      swi::launch_stencil_ds(P64, sb, sigt.as<double>(), c->stream, &c->launches);
+      swi::launch_stencil_ds(P64, reinterpret_cast<const double2*>(Vcur.p), ldv, reinterpret_cast<double2*>(Wblk.p),
+                             ldv, ncv, 1, sigt.as<double>(), c->pad_ds.as<float4>(), c->stream, &c->launches);
     } else {
       swi::launch_stencil_c64(P32, Vcur.as<float2>(), ldv, Wblk.as<float2>(), ldv, ncv, sigt.as<float>(),
                               c->stream, &c->launches);

@@ -88,7 +88,9 @@ struct StencilParams {
   double cm[7];       // -c_m / (2 h^2), m = 0..6 (centre weight counts once per axis)
   const double* V;    // N
   const double* G;    // Gamma_L + Gamma_R, N
+  const float4* VGds; // (V head, V tail, Gamma head, Gamma tail), N (the double-single kernel)
 };
+void launch_pack_vg_ds(const double* V, const double* G, long long n, float4* out, cudaStream_t s);
 
 // One block of columns for the batched stencil: Y[:, c] = (A - sigma[c]) X[:, c]
 struct StencilBlock {
@@ -96,7 +98,6 @@ struct StencilBlock {
   double2* Y;
   int ldx, ldy, ncols;
   int sigma_off;      // index into the sigma table of column 0
-  int out_ds;         // double-single kernel: Y holds (re hi, re lo, im hi, im lo) floats instead of complex128
 };
 
 // complex64 form (FP32 arithmetic), one block of columns
@@ -128,9 +129,13 @@ struct StencilBatch {
 
 void launch_stencil(const StencilParams& P, const StencilBatch& batch, const double* sigma_dev,
                     cudaStream_t s, long long* launches);
-// The same batched operator in double-single arithmetic (complex128 in and out).
-void launch_stencil_ds(const StencilParams& P, const StencilBatch& batch, const double* sigma_dev, cudaStream_t s,
-                       long long* launches);
+// The same operator on one block of columns in double-single arithmetic: X, Y
+// complex128 (Y four floats per entry, re hi, re lo, im hi, im lo, when out_ds),
+// sigma_dev one double per column; work of stencil_ds_work_bytes for the padded,
+// split copy of X.
+size_t stencil_ds_work_bytes(const StencilParams& P, int ncols);
+void launch_stencil_ds(const StencilParams& P, const double2* X, int ldx, double2* Y, int ldy, int ncols, int out_ds,
+                       const double* sigma_dev, float4* work, cudaStream_t s, long long* launches);
 
 // ---------------------------------------------------------------- tall-skinny products
 // C_j = op(X_j)^H diag(w) Y_j over the N rows (op = conj for the Hermitian
