@@ -21,11 +21,13 @@
 //
 //  sv_gram_kernel:   part[chunk][i][b] = sum_{rows of chunk} conj(Q[r, i]) w[r, b]
 //                    (a block per 32-column slab and row chunk, one column per lane)
-//  sv_update_kernel: w[r, :] -= Q[r, :] c (a warp per row), then the next
-//                    Gram's partials: one pass over Q for both (double-single)
+//  sv_update_kernel: w[r, :] -= Q[r, :] c, then the next Gram's partials: one
+//                    pass over Q for both (double-single)
 //  sv_update_fast_kernel: w[r, :] -= Q[r, :] c for the second pass's small
-//                    coefficients (FP32 products of the heads)
-//  sv_wgram_kernel:  part[chunk][a][b] = sum_{rows of chunk} conj(w[r, a]) w[r, b]
+//                    coefficients (FP32 products of the heads), then the
+//                    partials of w^H w
+//  sv_wgram_kernel:  part[chunk][a][b] = sum_{rows of chunk} conj(w[r, a]) w[r, b],
+//                    of a block as it is or times its Cholesky factor's inverse
 //  sv_reduce_kernel: FP64 sums of the chunk partials, added into columns of H;
 //                    for w^H w the Cholesky factor of the block (Cholesky-QR)
 // Chunks hold at most 1024 rows: the per-lane FP32 (or double-single) partial
@@ -60,28 +62,14 @@ struct PolC64 {
   using T = float2;   // basis element
   using A = float2;   // accumulator
   using S = float2;   // an element prepared for products (no split in FP32)
-  __device__ static S split(T v) { return v; }
-  __device__ static S bcast0(S v) {
-    return make_float2(__shfl_sync(0xffffffffu, v.x, 0), __shfl_sync(0xffffffffu, v.y, 0));
-  }
-  __device__ static void conj_mac_s(A& a, S q, S w) { conj_mac(a, q, w); }
-  __device__ static void mac_s(A& a, S q, S c) { mac(a, q, c); }
-  __device__ static A zero() { return make_float2(0.f, 0.f); }
   // a += conj(q) * w
   __device__ static void conj_mac(A& a, T q, T w) {
     a.x = fmaf(q.x, w.x, fmaf(q.y, w.y, a.x));
     a.y = fmaf(q.x, w.y, fmaf(-q.y, w.x, a.y));
   }
-  // a += q * c
-  __device__ static void mac(A& a, T q, T c) {
-    a.x = fmaf(q.x, c.x, fmaf(-q.y, c.y, a.x));
-    a.y = fmaf(q.x, c.y, fmaf(q.y, c.x, a.y));
-  }
-  __device__ static A add(A a, A b) { return make_float2(a.x + b.x, a.y + b.y); }
   __device__ static A shfl_xor(A a, int o) {
     return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
   }
-  __device__ static double2 to_d(A a) { return make_double2(a.x, a.y); }
   __device__ static T from_c(double2 c) { return make_float2((float)c.x, (float)c.y); }
   // the new vectors w: complex64, like the basis
   using W = float2;
@@ -89,27 +77,53 @@ struct PolC64 {
   __device__ static W wstore(S v) { return v; }
   __device__ static S wsub(S w, A d) { return make_float2(w.x - d.x, w.y - d.y); }
   __device__ static void gacc(Gds& g, S x, S y) { gds_acc(g, x.x, 0.f, x.y, 0.f, y.x, 0.f, y.y, 0.f); }
-  __device__ static double2 wto_d(W v) { return make_double2(v.x, v.y); }
-  __device__ static W wfrom_d(double2 v) { return make_float2((float)v.x, (float)v.y); }
+  __device__ static T out(S v) { return v; }  // a basis entry
   // the FP32 passes: the same arithmetic
   using F = float2;
   __device__ static F fzero() { return make_float2(0.f, 0.f); }
   __device__ static void fconj_mac(F& a, T q, S w) { conj_mac(a, q, w); }
-  __device__ static F fadd(F a, F b) { return add(a, b); }
-  __device__ static F fshfl_xor(F a, int o) { return shfl_xor(a, o); }
-  __device__ static double2 fto_d(F a) { return to_d(a); }
+  __device__ static F fadd(F a, F b) { return make_float2(a.x + b.x, a.y + b.y); }
+  __device__ static double2 fto_d(F a) { return make_double2(a.x, a.y); }
   __device__ static A fto_A(F a) { return a; }
   __device__ static float2 head2(T c) { return c; }
-  __device__ static void fmac2(F& a, T q, float2 c) { mac(a, q, c); }
+  // elements staged in shared memory for the accurate pass, and its accumulator
+  using ST = float2;
+  using AC = float2;
+  __host__ __device__ static int ldt(int ncols) { return (ncols + 15) / 16 * 16 + 8; }  // 8-byte rows: offset half a bank cycle
+  __device__ static ST stage(T v) { return v; }
+  static constexpr bool kStaged = true;  // a copied entry needs no conversion
+  __device__ static ST restage(ST v) { return v; }
+  __device__ static float2 raw_head(ST v) { return v; }
+  __device__ static ST swap(ST v) { return make_float2(v.y, v.x); }
+  __device__ static ST of_w(S v) { return v; }
+  __device__ static AC azero() { return make_float2(0.f, 0.f); }
+  __device__ static void tmac(AC& a, ST q, ST c, ST cs) {  // a += q c
+    a = __ffma2_rn(make_float2(q.x, q.x), c, a);
+    a = __ffma2_rn(make_float2(-q.y, q.y), cs, a);
+  }
+  __device__ static void tcmac(AC& a, ST q, ST w, ST wsw) {  // a += conj(q) w
+    a = __ffma2_rn(make_float2(q.x, q.x), w, a);
+    a = __ffma2_rn(make_float2(q.y, -q.y), wsw, a);
+  }
+  __device__ static AC tadd(AC a, AC b) { return __fadd2_rn(a, b); }
+  __device__ static AC tshx(AC a, int o) { return shfl_xor(a, o); }
+  __device__ static double2 tto_d(AC a) { return make_double2(a.x, a.y); }
+  __device__ static S wsub_t(S w, AC d) { return wsub(w, d); }
+  __device__ static S sshx(S a, int o) { return shfl_xor(a, o); }
+  __device__ static S smul2(S a, double2 r, S b, double2 t, bool two) {  // a r + b t, FP64 products
+    double re = a.x * r.x - a.y * r.y, im = a.x * r.y + a.y * r.x;
+    if (two) {
+      re += b.x * t.x - b.y * t.y;
+      im += b.x * t.y + b.y * t.x;
+    }
+    return make_float2((float)re, (float)im);
+  }
 };
 
-// x = hi + lo from the bit fields alone (integer and FP32 pipes only): hi is x
-// rounded to 24 significant bits, lo the remainder rounded to a float.  Values
-// below 2^-74 split to (0, 0) and magnitudes are capped at 2^126: the basis
-// entries, new vectors and coefficients of the loop lie far inside that range,
-// and no FP64 instruction is issued (a predicated FP64 fallback would occupy
-// GB300's narrow FP64 pipe on every element).
-__device__ __forceinline__ float hi_fast(double x) {  // the head of split_fast alone
+// Operands are split by ds::split_flush (no FP64 instruction on any path): the
+// basis entries, new vectors and coefficients of the loop lie far inside its
+// range.
+__device__ __forceinline__ float hi_fast(double x) {  // the head of ds::split_flush alone
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const unsigned int top = (unsigned int)(b >> 32);
   const int e0 = (int)((top >> 20) & 0x7ff);
@@ -117,21 +131,6 @@ __device__ __forceinline__ float hi_fast(double x) {  // the head of split_fast 
   const unsigned int fb =
       ((unsigned int)(e - 896) << 23 | ((unsigned int)(b >> 29) & 0x7fffffu)) + ((unsigned int)(b >> 28) & 1u);
   return e0 < 949 ? 0.f : __uint_as_float((top & 0x80000000u) | fb);
-}
-
-__device__ __forceinline__ void split_fast(double x, float& hi, float& lo) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const unsigned int top = (unsigned int)(b >> 32);
-  const unsigned int sgn = top & 0x80000000u;
-  const int e0 = (int)((top >> 20) & 0x7ff);
-  const bool small = e0 < 949;
-  const int e = min(max(e0, 949), 1149);
-  const unsigned int up = (unsigned int)(b >> 28) & 1u;
-  const unsigned int fb = ((unsigned int)(e - 896) << 23 | ((unsigned int)(b >> 29) & 0x7fffffu)) + up;
-  const int rem = (int)((unsigned int)b & 0x1fffffffu) - (int)(up << 29);
-  const float t = (float)rem * __uint_as_float((unsigned int)(e - 948) << 23);
-  hi = small ? 0.f : __uint_as_float(sgn | fb);
-  lo = small ? 0.f : (sgn ? -t : t);
 }
 
 struct PolDs {
@@ -142,41 +141,6 @@ struct PolDs {
   struct S {  // heads and tails of the real and imaginary parts
     float rh, rl, ih, il;
   };
-  __device__ static S split(T v) {
-    S o;
-    split_fast(v.x, o.rh, o.rl);
-    split_fast(v.y, o.ih, o.il);
-    return o;
-  }
-  __device__ static S bcast0(S v) {
-    return S{__shfl_sync(0xffffffffu, v.rh, 0), __shfl_sync(0xffffffffu, v.rl, 0), __shfl_sync(0xffffffffu, v.ih, 0),
-             __shfl_sync(0xffffffffu, v.il, 0)};
-  }
-  // a += conj(q) * w
-  __device__ static void conj_mac_s(A& a, const S& q, const S& w) {
-    ds::fma_acc(a.rh, a.re, q.rh, q.rl, w.rh, w.rl);
-    ds::fma_acc(a.rh, a.re, q.ih, q.il, w.ih, w.il);
-    ds::fma_acc(a.ih, a.ie, q.rh, q.rl, w.ih, w.il);
-    ds::fma_acc(a.ih, a.ie, -q.ih, -q.il, w.rh, w.rl);
-  }
-  // a += q * c
-  __device__ static void mac_s(A& a, const S& q, const S& c) {
-    ds::fma_acc(a.rh, a.re, q.rh, q.rl, c.rh, c.rl);
-    ds::fma_acc(a.rh, a.re, -q.ih, -q.il, c.ih, c.il);
-    ds::fma_acc(a.ih, a.ie, q.rh, q.rl, c.ih, c.il);
-    ds::fma_acc(a.ih, a.ie, q.ih, q.il, c.rh, c.rl);
-  }
-  __device__ static A zero() { return A{0.f, 0.f, 0.f, 0.f}; }
-  __device__ static A add(A a, A b) {
-    const ds::df r = ds::two_sum(a.rh, b.rh);
-    const ds::df i = ds::two_sum(a.ih, b.ih);
-    return A{r.h, r.l + a.re + b.re, i.h, i.l + a.ie + b.ie};
-  }
-  __device__ static A shfl_xor(A a, int o) {
-    return A{__shfl_xor_sync(0xffffffffu, a.rh, o), __shfl_xor_sync(0xffffffffu, a.re, o),
-             __shfl_xor_sync(0xffffffffu, a.ih, o), __shfl_xor_sync(0xffffffffu, a.ie, o)};
-  }
-  __device__ static double2 to_d(A a) { return make_double2((double)a.rh + (double)a.re, (double)a.ih + (double)a.ie); }
   __device__ static T from_c(double2 c) { return c; }
   // the new vectors w: kept in split form (heads and tails as floats) while
   // they are orthogonalised, so that forming w - Q c takes no FP64 instruction
@@ -189,12 +153,8 @@ struct PolDs {
     return S{r.h, r.l, i.h, i.l};
   }
   __device__ static void gacc(Gds& g, S x, S y) { gds_acc(g, x.rh, x.rl, x.ih, x.il, y.rh, y.rl, y.ih, y.il); }
-  __device__ static double2 wto_d(W v) { return make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w); }
-  __device__ static W wfrom_d(double2 v) {
-    S o;
-    split_fast(v.x, o.rh, o.rl);
-    split_fast(v.y, o.ih, o.il);
-    return wstore(o);
+  __device__ static T out(const S& v) {  // a basis entry (no FP64 instruction)
+    return make_double2(ds::join_bits(v.rh, v.rl), ds::join_bits(v.ih, v.il));
   }
   // the FP32 passes: products of the heads in FP32 (the first Gram of
   // classical Gram-Schmidt twice, and the update by the second pass's small
@@ -207,24 +167,109 @@ struct PolDs {
     a.y = fmaf(qr, w.ih, fmaf(-qi, w.rh, a.y));
   }
   __device__ static F fadd(F a, F b) { return make_float2(a.x + b.x, a.y + b.y); }
-  __device__ static F fshfl_xor(F a, int o) {
-    return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
-  }
   __device__ static double2 fto_d(F a) { return make_double2(a.x, a.y); }
   __device__ static A fto_A(F a) { return A{a.x, 0.f, a.y, 0.f}; }
   __device__ static float2 head2(T c) { return make_float2(hi_fast(c.x), hi_fast(c.y)); }
-  __device__ static void fmac2(F& a, T q, float2 c) {  // a += q c, FP32 products of the heads
-    const float qr = hi_fast(q.x), qi = hi_fast(q.y);
-    a.x = fmaf(qr, c.x, fmaf(-qi, c.y, a.x));
-    a.y = fmaf(qr, c.y, fmaf(qi, c.x, a.y));
+  // elements staged in shared memory for the accurate pass: heads (re, im), tails
+  // (re, im), so that real and imaginary parts go through packed FP32x2
+  // instructions; the accumulator likewise
+  using ST = float4;
+  struct AC {
+    float2 h, l;
+  };
+  __host__ __device__ static int ldt(int ncols) { return ncols; }
+  __device__ static ST stage(T v) {
+    ST o;
+    ds::split_flush(v.x, o.x, o.z);
+    ds::split_flush(v.y, o.y, o.w);
+    return o;
+  }
+  static constexpr bool kStaged = false;
+  // an entry as copied (the bytes of a T)
+  __device__ static T raw(ST v) {
+    return make_double2(__hiloint2double(__float_as_int(v.y), __float_as_int(v.x)),
+                        __hiloint2double(__float_as_int(v.w), __float_as_int(v.z)));
+  }
+  __device__ static ST restage(ST v) { return stage(raw(v)); }
+  __device__ static float2 raw_head(ST v) { return head2(raw(v)); }
+  __device__ static ST swap(ST v) { return make_float4(v.y, v.x, v.w, v.z); }
+  __device__ static ST of_w(const S& v) { return make_float4(v.rh, v.ih, v.rl, v.il); }
+  __device__ static AC azero() { return AC{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
+  __device__ static float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+  // a += (uh + ul) (vh + vl) per component: exact product up to its tail, head by
+  // TwoSum; nh = -uh, so that the product arrives negated and no operand of a
+  // packed instruction needs its sign turned
+  __device__ static void mulv(AC& a, float2 uh, float2 nh, float2 ul, float2 vh, float2 vl) {
+    const float2 np = __fmul2_rn(nh, vh);
+    float2 e = __ffma2_rn(uh, vh, np);
+    e = __ffma2_rn(uh, vl, e);
+    e = __ffma2_rn(ul, vh, e);
+    const float2 t = sub2(a.h, np);
+    const float2 bp = sub2(t, a.h);
+    const float2 err = sub2(sub2(a.h, sub2(t, bp)), __fadd2_rn(np, bp));
+    a.h = t;
+    a.l = __fadd2_rn(a.l, __fadd2_rn(err, e));
+  }
+  __device__ static void tmac(AC& a, ST q, ST c, ST cs) {  // a += q c
+    mulv(a, make_float2(q.x, q.x), make_float2(-q.x, -q.x), make_float2(q.z, q.z), make_float2(c.x, c.y),
+         make_float2(c.z, c.w));
+    mulv(a, make_float2(-q.y, q.y), make_float2(q.y, -q.y), make_float2(-q.w, q.w), make_float2(cs.x, cs.y),
+         make_float2(cs.z, cs.w));
+  }
+  __device__ static void tcmac(AC& a, ST q, ST w, ST wsw) {  // a += conj(q) w
+    mulv(a, make_float2(q.x, q.x), make_float2(-q.x, -q.x), make_float2(q.z, q.z), make_float2(w.x, w.y),
+         make_float2(w.z, w.w));
+    mulv(a, make_float2(q.y, -q.y), make_float2(-q.y, q.y), make_float2(q.w, -q.w), make_float2(wsw.x, wsw.y),
+         make_float2(wsw.z, wsw.w));
+  }
+  __device__ static AC tadd(AC a, AC b) {
+    const float2 t = __fadd2_rn(a.h, b.h);
+    const float2 bp = sub2(t, a.h);
+    const float2 err = __fadd2_rn(sub2(a.h, sub2(t, bp)), sub2(b.h, bp));
+    return AC{t, __fadd2_rn(__fadd2_rn(a.l, b.l), err)};
+  }
+  __device__ static float2 sx(float2 a, int o) {
+    return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
+  }
+  __device__ static AC tshx(AC a, int o) { return AC{sx(a.h, o), sx(a.l, o)}; }
+  __device__ static double2 tto_d(AC a) {
+    return make_double2((double)a.h.x + (double)a.l.x, (double)a.h.y + (double)a.l.y);
+  }
+  __device__ static S sshx(const S& a, int o) {
+    const float2 r = sx(make_float2(a.rh, a.rl), o), i = sx(make_float2(a.ih, a.il), o);
+    return S{r.x, r.y, i.x, i.y};
+  }
+  __device__ static S wsub_t(const S& w, AC d) { return wsub(w, A{d.h.x, d.l.x, d.h.y, d.l.y}); }
+  __device__ static S smul2(const S& a, double2 r, const S& b, double2 t, bool two) {  // a r + b t in double-single
+    const ST rs = stage(r), ts = stage(t);
+    AC s = azero();
+    tmac(s, of_w(a), rs, swap(rs));
+    if (two) tmac(s, of_w(b), ts, swap(ts));
+    const ds::df x = ds::two_sum(s.h.x, s.l.x), y = ds::two_sum(s.h.y, s.l.y);
+    return S{x.h, x.l, y.h, y.l};
   }
 };
 
+// a basis entry (8 or 16 bytes) from global to shared memory, asynchronously; zero if !on
+template <class ST>
+__device__ __forceinline__ void copy_entry(ST* dst, const ST* src, bool on) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  const int n = on ? (int)sizeof(ST) : 0;
+  if constexpr (sizeof(ST) == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copies_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // ----------------------------------------------------------------- Gram pass
-template <class Pol, int NB, bool FAST>
+template <class Pol, int NB>
 __global__ void __launch_bounds__(kThreads) sv_gram_kernel(const __grid_constant__ SvBatch batch, int N, int rpc) {
   using T = typename Pol::T;
-  using A = typename Pol::A;
   const SvJob& J = batch.job[blockIdx.z];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int col = blockIdx.y * 32 + lane;
@@ -236,51 +281,28 @@ __global__ void __launch_bounds__(kThreads) sv_gram_kernel(const __grid_constant
   const bool on = col < J.ncols;
   __shared__ double2 red[kWarps][NB][32];
   int r = r0 + warp;
-  if constexpr (FAST) {
-    // four rows per iteration, their loads issued together (memory-level
-    // parallelism), two interleaved accumulators per column of w
-    typename Pol::F a0[NB], a1[NB];
+  // four rows per iteration, their loads issued together (memory-level
+  // parallelism), two interleaved accumulators per column of w
+  typename Pol::F a0[NB], a1[NB];
 #pragma unroll
-    for (int b = 0; b < NB; ++b) a0[b] = a1[b] = Pol::fzero();
-    for (; r + 3 * kWarps < r1; r += 4 * kWarps) {
-      T q[4];
+  for (int b = 0; b < NB; ++b) a0[b] = a1[b] = Pol::fzero();
+  for (; r + 3 * kWarps < r1; r += 4 * kWarps) {
+    T q[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) q[u] = on ? __ldg(Q + (long long)(r + u * kWarps) * J.ldq + col) : T{};
+    for (int u = 0; u < 4; ++u) q[u] = on ? __ldg(Q + (long long)(r + u * kWarps) * J.ldq + col) : T{};
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int b = 0; b < NB; ++b)
-          Pol::fconj_mac((u & 1) ? a1[b] : a0[b], q[u], Pol::wload(w[(long long)(r + u * kWarps) * J.ldw + b]));
-    }
-    for (; r < r1; r += kWarps) {
-      const T q0 = on ? __ldg(Q + (long long)r * J.ldq + col) : T{};
-#pragma unroll
-      for (int b = 0; b < NB; ++b) Pol::fconj_mac(a0[b], q0, Pol::wload(w[(long long)r * J.ldw + b]));
-    }
-#pragma unroll
-    for (int b = 0; b < NB; ++b) red[warp][b][lane] = Pol::fto_d(Pol::fadd(a0[b], a1[b]));
-  } else {
-    A a0[NB], a1[NB];
-#pragma unroll
-    for (int b = 0; b < NB; ++b) a0[b] = a1[b] = Pol::zero();
-    for (; r + kWarps < r1; r += 2 * kWarps) {
-      const T q0 = on ? __ldg(Q + (long long)r * J.ldq + col) : T{};
-      const T q1 = on ? __ldg(Q + (long long)(r + kWarps) * J.ldq + col) : T{};
-      const auto s0 = Pol::split(q0), s1 = Pol::split(q1);
-#pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        Pol::conj_mac_s(a0[b], s0, Pol::wload(w[(long long)r * J.ldw + b]));
-        Pol::conj_mac_s(a1[b], s1, Pol::wload(w[(long long)(r + kWarps) * J.ldw + b]));
-      }
-    }
-    if (r < r1) {
-      const auto s0 = Pol::split(on ? __ldg(Q + (long long)r * J.ldq + col) : T{});
-#pragma unroll
-      for (int b = 0; b < NB; ++b) Pol::conj_mac_s(a0[b], s0, Pol::wload(w[(long long)r * J.ldw + b]));
-    }
-#pragma unroll
-    for (int b = 0; b < NB; ++b) red[warp][b][lane] = Pol::to_d(Pol::add(a0[b], a1[b]));
+      for (int b = 0; b < NB; ++b)
+        Pol::fconj_mac((u & 1) ? a1[b] : a0[b], q[u], Pol::wload(w[(long long)(r + u * kWarps) * J.ldw + b]));
   }
+  for (; r < r1; r += kWarps) {
+    const T q0 = on ? __ldg(Q + (long long)r * J.ldq + col) : T{};
+#pragma unroll
+    for (int b = 0; b < NB; ++b) Pol::fconj_mac(a0[b], q0, Pol::wload(w[(long long)r * J.ldw + b]));
+  }
+#pragma unroll
+  for (int b = 0; b < NB; ++b) red[warp][b][lane] = Pol::fto_d(Pol::fadd(a0[b], a1[b]));
   __syncthreads();
   if (warp == 0 && on) {
 #pragma unroll
@@ -298,174 +320,313 @@ __global__ void __launch_bounds__(kThreads) sv_gram_kernel(const __grid_constant
 
 // ----------------------------------------------------------------- update fused with the second Gram
 // The accurate pass: w[r, :] -= Q[r, :] c, then the partials of Q^H w, in
-// double-single.  A warp per row; lane l holds basis columns l, l + 32, ...
-// (NT of them); the row's values are read twice (the second read hits L1)
-// rather than held in registers, which keeps two blocks on an SM.
-template <class Pol, int NT, int NB>
-__global__ void __launch_bounds__(kThreads, (NT <= 8) ? 2 : 1) sv_update_kernel(const __grid_constant__ SvBatch batch, int N, int rpc) {
+// double-single (FP32 in the complex64 form).  A tile of RT rows is staged once
+// in shared memory, split into heads and tails as it arrives; the update then
+// gives each row to 256 / RT lanes (three to five shuffle levels per row), the
+// Gram gives each column to a thread (to 256 / columns row groups when there
+// are fewer than 256), which needs no shuffles and no accumulators beyond its
+// own column's.  FP32 issue bounds it (192 operations per basis entry at
+// nb = 2, half the issue slots when packed), so every entry is split once.
+// Measured with its reduction (one window of 48x48x96, ~58 to 116 columns, nb = 2):
+// 306 us (354 alone at 116 columns: 59% of the issue slots); a warp per
+// row with both products from global memory, splitting twice and reducing over
+// 32 lanes, took 459 us (2,000 rows in four windows: 112 us, now 24).
+template <class Pol, int RT, int NC2, int NB, int NBUF>
+__global__ void __launch_bounds__(kThreads, NC2 == 1 ? 3 : 1)
+    sv_update_kernel(const __grid_constant__ SvBatch batch, int N, int rpc) {
   using T = typename Pol::T;
-  using A = typename Pol::A;
+  using ST = typename Pol::ST;
+  using AC = typename Pol::AC;
   using Sp = typename Pol::S;
-  // shared: the coefficients c in split form, then the cross-warp partials
-  extern __shared__ double2 sh[];
-  const SvJob& J = batch.job[blockIdx.y];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int ncols = J.ncols;
-  Sp* cs = reinterpret_cast<Sp*>(sh);
-  double2* red = sh + (size_t)ncols * NB;
-  // stored vector-major (cs[b * ncols + i]): a warp's lanes read consecutive
-  // 16-byte entries, without bank conflicts
-  for (int e = threadIdx.x; e < ncols * NB; e += kThreads) cs[(e % NB) * ncols + e / NB] = Pol::split(Pol::from_c(J.c[e]));
-  __syncthreads();
   using Wt = typename Pol::W;
-  const T* __restrict__ Q = static_cast<const T*>(J.Q);
+  constexpr int L = kThreads / RT;  // lanes per row of the update
+  static_assert(L <= 32, "a row's lanes lie in one warp");
+  extern __shared__ __align__(16) unsigned char raw[];
+  const SvJob& J = batch.job[blockIdx.y];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ncols = J.ncols, ldt = Pol::ldt(ncols);
+  ST* cs = reinterpret_cast<ST*>(raw);  // coefficients [NB][2][ncols]: as they are, parts swapped
+  ST* ws = cs + NB * 2 * ncols;         // the tile's new values [RT][NB][2]
+  ST* tile = ws + RT * NB * 2;          // [NBUF][RT][ldt]
+  for (int e = tid; e < ncols * NB; e += kThreads) {
+    const ST v = Pol::stage(Pol::from_c(J.c[e]));
+    cs[(e % NB) * 2 * ncols + e / NB] = v;
+    cs[((e % NB) * 2 + 1) * ncols + e / NB] = Pol::swap(v);
+  }
+  const ST* __restrict__ Q = static_cast<const ST*>(J.Q);  // entries as bytes
   Wt* w = static_cast<Wt*>(J.w);
   const int r0 = blockIdx.x * rpc, r1 = min(N, r0 + rpc);
-  A acc[NT][NB];
+  // Gram role: column(s) gcol, gcol + 256, ..., rows g, g + G, ...
+  const int cpad = min(kThreads, (ncols + 31) & ~31), G = kThreads / cpad;
+  const int g = tid / cpad, gcol = tid - g * cpad;
+  AC acc[NC2][NB];
 #pragma unroll
-  for (int t = 0; t < NT; ++t)
+  for (int k = 0; k < NC2; ++k)
 #pragma unroll
-    for (int b = 0; b < NB; ++b) acc[t][b] = Pol::zero();
-  for (int r = r0 + warp; r < r1; r += kWarps) {
-    // Q[r, :] c, two interleaved accumulators per new vector (independent chains)
-    A d[NB], d1[NB];
+    for (int b = 0; b < NB; ++b) acc[k][b] = Pol::azero();
+  const auto fetch = [&](int rb, ST* dst) {
 #pragma unroll
-    for (int b = 0; b < NB; ++b) d[b] = d1[b] = Pol::zero();
+    for (int k = 0; k < RT / kWarps; ++k) {
+      const int r = warp + k * kWarps, row = rb + r;
+      const bool on = row < r1;
+      const ST* src = Q + (long long)(on ? row : r0) * J.ldq;
+      for (int i = lane; i < ncols; i += 32) copy_entry(dst + r * ldt + i, src + i, on);
+    }
+    copies_commit();
+  };
+  ST* const first = tile;
+  fetch(r0, tile);
+  for (int rb = r0; rb < r1; rb += RT) {
+    copies_wait<0>();
+    if constexpr (!Pol::kStaged) {  // every thread converts, in place, what it copied
 #pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      const int i = lane + 32 * t;
-      if (i < ncols) {
-        const Sp qs = Pol::split(__ldg(Q + (long long)r * J.ldq + i));
-#pragma unroll
-        for (int b = 0; b < NB; ++b) Pol::mac_s((t & 1) ? d1[b] : d[b], qs, cs[b * ncols + i]);
+      for (int k = 0; k < RT / kWarps; ++k) {
+        ST* t = tile + (warp + k * kWarps) * ldt;
+#pragma unroll 4
+        for (int i = lane; i < ncols; i += 32) t[i] = Pol::restage(t[i]);
       }
     }
+    __syncthreads();  // the tile is there, and the last one's products are done
+    if (NBUF == 2 && rb + RT < r1) fetch(rb + RT, tile == first ? first + RT * ldt : first);
+    {
+      const int r = tid / L, sub = tid % L, row = rb + r;
+      AC d[NB];
 #pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      d[b] = Pol::add(d[b], d1[b]);
+      for (int b = 0; b < NB; ++b) d[b] = Pol::azero();
+      for (int i = sub; i < ncols; i += L) {
+        const ST q = tile[r * ldt + i];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) d[b] = Pol::add(d[b], Pol::shfl_xor(d[b], o));
-    }
-    // the row's new values are formed by lane 0 alone (FP32 instructions
-    // only, in split form) and broadcast
-    Sp ws[NB]{};
-    if (lane == 0) {
-#pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        ws[b] = Pol::wsub(Pol::wload(w[(long long)r * J.ldw + b]), d[b]);
-        w[(long long)r * J.ldw + b] = Pol::wstore(ws[b]);
+        for (int b = 0; b < NB; ++b) Pol::tmac(d[b], q, cs[2 * b * ncols + i], cs[(2 * b + 1) * ncols + i]);
       }
-    }
 #pragma unroll
-    for (int b = 0; b < NB; ++b) ws[b] = Pol::bcast0(ws[b]);
+      for (int b = 0; b < NB; ++b)
 #pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      const int i = lane + 32 * t;
-      if (i < ncols) {
-        const Sp qs = Pol::split(__ldg(Q + (long long)r * J.ldq + i));
+        for (int o = L / 2; o > 0; o >>= 1) d[b] = Pol::tadd(d[b], Pol::tshx(d[b], o));
+      // lane b of the row forms the row's new value of vector b
 #pragma unroll
-        for (int b = 0; b < NB; ++b) Pol::conj_mac_s(acc[t][b], qs, ws[b]);
-      }
-    }
-  }
-  double2* out = J.part + (long long)blockIdx.x * J.ldp;
-  // cross-warp sums, one 32-column slab at a time: red [kWarps][NB][32]
-#pragma unroll
-  for (int t = 0; t < NT; ++t) {
-    if (32 * t >= ncols) break;  // uniform over the block
-#pragma unroll
-    for (int b = 0; b < NB; ++b) red[(warp * NB + b) * 32 + lane] = Pol::to_d(acc[t][b]);
-    __syncthreads();
-    if (threadIdx.x < 32 * NB) {
-      const int b = threadIdx.x >> 5, l = threadIdx.x & 31, i = l + 32 * t;
-      if (i < ncols) {
-        double2 s = make_double2(0.0, 0.0);
-        for (int k = 0; k < kWarps; ++k) {
-          s.x += red[(k * NB + b) * 32 + l].x;
-          s.y += red[(k * NB + b) * 32 + l].y;
+      for (int b = 0; b < NB; ++b)
+        if (sub == b) {
+          Sp v{};
+          if (row < r1) {
+            v = Pol::wsub_t(Pol::wload(w[(long long)row * J.ldw + b]), d[b]);
+            w[(long long)row * J.ldw + b] = Pol::wstore(v);
+          }
+          const ST t = Pol::of_w(v);
+          ws[(r * NB + b) * 2] = t;
+          ws[(r * NB + b) * 2 + 1] = Pol::swap(t);
         }
-        out[i * NB + b] = s;
-      }
     }
     __syncthreads();
-  }
-}
-
-// ----------------------------------------------------------------- the second update (FP32 products)
-// w[r, :] -= Q[r, :] c for the second pass's small coefficients: products of
-// the basis heads in FP32, the row's new value formed in split form by lane 0;
-// a warp per row, few registers so that four blocks share an SM.
-template <class Pol, int NT, int NB>
-__global__ void __launch_bounds__(kThreads, (NT <= 8) ? 4 : ((NT <= 12) ? 2 : 1)) sv_update_fast_kernel(const __grid_constant__ SvBatch batch, int N,
-                                                                      int rpc) {
-  using T = typename Pol::T;
-  using F = typename Pol::F;
-  using Sp = typename Pol::S;
-  using Wt = typename Pol::W;
-  extern __shared__ double2 sh[];
-  const SvJob& J = batch.job[blockIdx.y];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int ncols = J.ncols;
-  // the coefficients' heads, [NB][ncols] (8 bytes per entry: conflict-free reads)
-  float2* cs = reinterpret_cast<float2*>(sh);
-  for (int e = threadIdx.x; e < ncols * NB; e += kThreads) cs[(e % NB) * ncols + e / NB] = Pol::head2(Pol::from_c(J.c[e]));
-  __syncthreads();
-  const T* __restrict__ Q = static_cast<const T*>(J.Q);
-  Wt* w = static_cast<Wt*>(J.w);
-  const int r0 = blockIdx.x * rpc, r1 = min(N, r0 + rpc);
-  constexpr int kRows = 1;
-  for (int r = r0 + warp; r < r1; r += kRows * kWarps) {
-    const int rb = r + kWarps;
-    const bool two = kRows == 2 && rb < r1;
-    T qa[NT], qb[kRows == 2 ? NT : 1];
+    if (g < G) {
+#pragma unroll 2
+      for (int r = g; r < RT; r += G) {
 #pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      const int i = lane + 32 * t;
-      qa[t] = i < ncols ? __ldg(Q + (long long)r * J.ldq + i) : T{};
-      if (kRows == 2) qb[kRows == 2 ? t : 0] = (two && i < ncols) ? __ldg(Q + (long long)rb * J.ldq + i) : T{};
+        for (int k = 0; k < NC2; ++k) {
+          const int i = gcol + k * kThreads;
+          if (i < ncols) {
+            const ST q = tile[r * ldt + i];
+#pragma unroll
+            for (int b = 0; b < NB; ++b) Pol::tcmac(acc[k][b], q, ws[(r * NB + b) * 2], ws[(r * NB + b) * 2 + 1]);
+          }
+        }
+      }
     }
-    F fa[NB], fb[NB];
+    if (NBUF == 2) {
+      tile = tile == first ? first + RT * ldt : first;
+    } else {
+      __syncthreads();
+      if (rb + RT < r1) fetch(rb + RT, tile);
+    }
+  }
+  __syncthreads();
+  // sums of the row groups (the tile's space holds them; G > 1 only with one column per thread)
+  double2* out = J.part + (long long)blockIdx.x * J.ldp;
+  double2* red = reinterpret_cast<double2*>(raw);
+  if (G > 1) {
+    if (g > 0 && g < G && gcol < ncols)
 #pragma unroll
-    for (int b = 0; b < NB; ++b) fa[b] = fb[b] = Pol::fzero();
+      for (int b = 0; b < NB; ++b) red[((g - 1) * NB + b) * cpad + gcol] = Pol::tto_d(acc[0][b]);
+    __syncthreads();
+  }
+  if (g == 0) {
 #pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      const int i = lane + 32 * t;
+    for (int k = 0; k < NC2; ++k) {
+      const int i = gcol + k * kThreads;
       if (i < ncols)
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
-          const float2 cv = cs[b * ncols + i];
-          Pol::fmac2(fa[b], qa[t], cv);
-          if (kRows == 2) Pol::fmac2(fb[b], qb[kRows == 2 ? t : 0], cv);
+          double2 s = Pol::tto_d(acc[k][b]);
+          for (int q = 1; q < G; ++q) {
+            const double2 v = red[((q - 1) * NB + b) * cpad + i];
+            s.x += v.x;
+            s.y += v.y;
+          }
+          out[i * NB + b] = s;
         }
     }
+  }
+}
+
+// sum over a block of the NB x NB entries held (as FP64) by its threads, into
+// out[0 .. NB NB); red: [kWarps][NB * NB]
+template <int NB>
+__device__ __forceinline__ void block_sum_small(const Gds* g, double2 (*red)[NB * NB], double2* out) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int b = 0; b < NB; ++b)
+  for (int e = 0; e < NB * NB; ++e) {
+    double2 s = make_double2((double)g[e].rh + (double)g[e].re, (double)g[e].ih + (double)g[e].ie);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        fa[b] = Pol::fadd(fa[b], Pol::fshfl_xor(fa[b], o));
-        fb[b] = Pol::fadd(fb[b], Pol::fshfl_xor(fb[b], o));
+    for (int o = 16; o > 0; o >>= 1) {
+      s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+      s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+    }
+    if (lane == 0) red[warp][e] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x < NB * NB) {
+    double2 s = red[0][threadIdx.x];
+#pragma unroll
+    for (int k = 1; k < kWarps; ++k) {
+      s.x += red[k][threadIdx.x].x;
+      s.y += red[k][threadIdx.x].y;
+    }
+    out[threadIdx.x] = s;
+  }
+}
+
+// ----------------------------------------------------------------- the second update (FP32 products) and w^H w
+// w[r, :] -= Q[r, :] c for the second pass's small coefficients: products of
+// the basis heads in FP32; and the new block's Gram matrix in double-single on
+// the way.  HBM-bound: a warp takes R rows at a time and copies the next R into
+// its half of shared memory meanwhile (every lane reads only what it copied, so
+// nothing waits on another lane); the R x NB products are summed over the lanes
+// by halving - every level keeps half the values per lane - so that
+// R NB + log2(32 / (R NB)) exchanges serve all of them; then each value's first
+// lane forms the row's new entry.
+template <class Pol, int NB, int R>
+__global__ void __launch_bounds__(kThreads)
+    sv_update_fast_kernel(const __grid_constant__ SvBatch batch, int N, int rpc, int stages) {
+  using ST = typename Pol::ST;
+  using Sp = typename Pol::S;
+  using Wt = typename Pol::W;
+  constexpr int V = R * NB;  // values per warp pass, index row * NB + b
+  extern __shared__ __align__(16) unsigned char raw[];
+  __shared__ double2 red[kWarps][NB * NB];
+  const SvJob& J = batch.job[blockIdx.y];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int ncols = J.ncols;
+  ST* ring = reinterpret_cast<ST*>(raw) + (size_t)warp * stages * R * ncols;  // [stages][R][ncols] per warp
+  // the coefficients' heads, [NB][ncols] (8 bytes per entry: conflict-free reads)
+  float2* cs = reinterpret_cast<float2*>(reinterpret_cast<ST*>(raw) + (size_t)kWarps * stages * R * ncols);
+  const ST* __restrict__ Q = static_cast<const ST*>(J.Q);  // entries as bytes
+  Wt* w = static_cast<Wt*>(J.w);
+  const int r0 = blockIdx.x * rpc, r1 = min(N, r0 + rpc);
+  const auto fetch = [&](int r, ST* dst) {
+#pragma unroll
+    for (int u = 0; u < R; ++u) {
+      const bool on = r + u < r1;
+      const ST* src = Q + (long long)(on ? r + u : r0) * J.ldq;
+      for (int i = lane; i < ncols; i += 32) copy_entry(dst + u * ncols + i, src + i, on);
+    }
+  };
+  int st = 0;
+  if (r0 + warp * R < r1) fetch(r0 + warp * R, ring);
+  copies_commit();
+  for (int e = threadIdx.x; e < ncols * NB; e += kThreads) cs[(e % NB) * ncols + e / NB] = Pol::head2(Pol::from_c(J.c[e]));
+  __syncthreads();
+  constexpr int kLow = 32 / V;  // lanes left per value
+  const int vi = lane / kLow, vrow = vi / NB, vb = vi % NB;
+  Gds g[NB * NB];
+#pragma unroll
+  for (int e = 0; e < NB * NB; ++e) g[e] = Gds{0.f, 0.f, 0.f, 0.f};
+  for (int r = r0 + warp * R; r < r1; r += kWarps * R) {
+    const int rn = r + kWarps * R;
+    if (stages == 2) {
+      if (rn < r1) fetch(rn, ring + (st ^ 1) * R * ncols);
+      copies_commit();
+      copies_wait<1>();
+    } else {
+      copies_wait<0>();
+    }
+    const ST* q = ring + st * R * ncols;
+    // the value this lane will finish: its old entry, loaded beside the basis
+    const bool on = r + vrow < r1;
+    Wt* wp = w + (long long)(r + vrow) * J.ldw + vb;
+    Sp old{};
+    if (on) old = Pol::wload(*wp);
+    float2 f[V];
+#pragma unroll
+    for (int e = 0; e < V; ++e) f[e] = make_float2(0.f, 0.f);
+#pragma unroll 2
+    for (int i = lane; i < ncols; i += 32) {
+      float2 c[NB];
+#pragma unroll
+      for (int b = 0; b < NB; ++b) c[b] = cs[b * ncols + i];
+#pragma unroll
+      for (int u = 0; u < R; ++u) {
+        const float2 h = Pol::raw_head(q[u * ncols + i]);
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+          float2& a = f[u * NB + b];
+          a.x = fmaf(h.x, c[b].x, fmaf(-h.y, c[b].y, a.x));
+          a.y = fmaf(h.x, c[b].y, fmaf(h.y, c[b].x, a.y));
+        }
       }
-    if (lane == 0) {
+    }
+    if (stages == 2) {
+      st ^= 1;
+    } else {
+      if (rn < r1) fetch(rn, ring);
+      copies_commit();
+    }
 #pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        w[(long long)r * J.ldw + b] = Pol::wstore(Pol::wsub(Pol::wload(w[(long long)r * J.ldw + b]), Pol::fto_A(fa[b])));
-        if (two)
-          w[(long long)rb * J.ldw + b] =
-              Pol::wstore(Pol::wsub(Pol::wload(w[(long long)rb * J.ldw + b]), Pol::fto_A(fb[b])));
+    for (int n = V / 2, o = 16; n > 0; n >>= 1, o >>= 1) {
+      const bool up = lane & o;
+#pragma unroll
+      for (int e = 0; e < n; ++e) {
+        const float2 keep = up ? f[e + n] : f[e], give = up ? f[e] : f[e + n];
+        f[e].x = keep.x + __shfl_xor_sync(0xffffffffu, give.x, o);
+        f[e].y = keep.y + __shfl_xor_sync(0xffffffffu, give.y, o);
+      }
+    }
+#pragma unroll
+    for (int o = kLow / 2; o > 0; o >>= 1) {
+      f[0].x += __shfl_xor_sync(0xffffffffu, f[0].x, o);
+      f[0].y += __shfl_xor_sync(0xffffffffu, f[0].y, o);
+    }
+    const Sp v = Pol::wsub(old, Pol::fto_A(f[0]));
+    const bool own = on && lane % kLow == 0;
+    if (own) *wp = Pol::wstore(v);
+    if constexpr (NB == 1) {
+      if (own) Pol::gacc(g[0], v, v);
+    } else {
+      const Sp v1 = Pol::sshx(v, kLow);  // the row's other vector
+      if (own && vb == 0) {
+        Pol::gacc(g[0], v, v);
+        Pol::gacc(g[1], v, v1);
+        Pol::gacc(g[2], v1, v);
+        Pol::gacc(g[3], v1, v1);
       }
     }
   }
+  block_sum_small<NB>(g, red, J.part + (long long)blockIdx.x * J.ldp);
 }
 
 // ----------------------------------------------------------------- w^H w of the new block
 // A block per row chunk and job, a thread per row (strided): double-single
-// products on every lane, FP64 sums across the block.
-template <class Pol, int NB>
+// products on every lane, FP64 sums across the block.  With r set the row is
+// first multiplied by the Cholesky factor's inverse (in place): the first
+// normalisation of a 2-vector block with the Gram matrix of the second.
+template <class Pol, int NB, bool SCALE>
 __global__ void __launch_bounds__(kThreads) sv_wgram_kernel(const __grid_constant__ SvBatch batch, int N, int rpc) {
   using Wt = typename Pol::W;
   const SvJob& J = batch.job[blockIdx.y];
-  const Wt* __restrict__ w = static_cast<const Wt*>(J.w);
+  Wt* w = static_cast<Wt*>(J.w);
   const int r0 = blockIdx.x * rpc, r1 = min(N, r0 + rpc);
+  __shared__ double2 red[kWarps][NB * NB];
+  double2 ri[NB * NB];
+#pragma unroll
+  for (int e = 0; e < NB * NB; ++e) ri[e] = SCALE ? J.c[e] : make_double2(0.0, 0.0);
   Gds g[NB * NB];
 #pragma unroll
   for (int e = 0; e < NB * NB; ++e) g[e] = Gds{0.f, 0.f, 0.f, 0.f};
@@ -473,32 +634,31 @@ __global__ void __launch_bounds__(kThreads) sv_wgram_kernel(const __grid_constan
     typename Pol::S v[NB];
 #pragma unroll
     for (int b = 0; b < NB; ++b) v[b] = Pol::wload(w[(long long)r * J.ldw + b]);
+    if constexpr (SCALE) {
+      typename Pol::S o[NB];
+#pragma unroll
+      for (int b = 0; b < NB; ++b) {  // column b of v R^-1 (upper triangular)
+        o[b] = Pol::smul2(v[0], ri[b], v[NB - 1], ri[(NB - 1) * NB + b], b > 0);
+        w[(long long)r * J.ldw + b] = Pol::wstore(o[b]);
+      }
+#pragma unroll
+      for (int b = 0; b < NB; ++b) v[b] = o[b];
+    }
 #pragma unroll
     for (int a = 0; a < NB; ++a)
 #pragma unroll
       for (int b = 0; b < NB; ++b) Pol::gacc(g[a * NB + b], v[a], v[b]);
   }
-  __shared__ double2 red[NB * NB][kThreads];
-#pragma unroll
-  for (int e = 0; e < NB * NB; ++e)
-    red[e][threadIdx.x] = make_double2((double)g[e].rh + (double)g[e].re, (double)g[e].ih + (double)g[e].ie);
-  __syncthreads();
-  for (int st = kThreads / 2; st > 0; st >>= 1) {
-    if ((int)threadIdx.x < st)
-#pragma unroll
-      for (int e = 0; e < NB * NB; ++e) {
-        red[e][threadIdx.x].x += red[e][threadIdx.x + st].x;
-        red[e][threadIdx.x].y += red[e][threadIdx.x + st].y;
-      }
-    __syncthreads();
-  }
-  if (threadIdx.x < NB * NB) J.part[(long long)blockIdx.x * J.ldp + threadIdx.x] = red[threadIdx.x][0];
+  block_sum_small<NB>(g, red, J.part + (long long)blockIdx.x * J.ldp);
 }
 
 // ----------------------------------------------------------------- chunk reduction
-// A block per 32 entries and job; 32 lanes per entry step through the chunks
-// (independent loads in flight), then combine in shared memory.
-constexpr int kRedLanes = 32;
+// A block per 8 entries and job (per 4 entries where the block's Gram matrix is
+// summed): the FP64 additions bound it, and a warp instruction takes ~19 cycles of
+// an SM's FP64 pipe however few lanes are on, so the entries are spread over
+// many SMs and every warp's lanes filled with (entry, chunk) pairs.  With 32
+// entries and 1024 threads to a block it took 16 us cold, now 9.
+constexpr int kRedThreads = 256;
 
 // upper Cholesky factor R of the Hermitian nb x nb matrix G (G = R^H R), its
 // inverse, and whether a pivot fell below 1e-14 of its diagonal entry
@@ -507,11 +667,11 @@ __device__ bool chol_small(const double2* G, int nb, double2* R, double2* Ri) {
   for (int e = 0; e < 4; ++e) R[e] = Ri[e] = make_double2(0.0, 0.0);
   const double g00 = G[0].x;
   if (!(g00 > 0.0)) return true;
-  const double r00 = sqrt(g00);
+  const double r00 = sqrt(g00), i00 = 1.0 / r00;
   R[0] = make_double2(r00, 0.0);
-  Ri[0] = make_double2(1.0 / r00, 0.0);
+  Ri[0] = make_double2(i00, 0.0);
   if (nb == 1) return false;
-  const double2 r01 = make_double2(G[1].x / r00, G[1].y / r00);
+  const double2 r01 = make_double2(G[1].x * i00, G[1].y * i00);
   const double d = G[3].x - (r01.x * r01.x + r01.y * r01.y);
   if (!(d > 1e-14 * G[3].x)) {
     bad = true;
@@ -520,24 +680,26 @@ __device__ bool chol_small(const double2* G, int nb, double2* R, double2* Ri) {
   R[1] = r01;
   R[3] = make_double2(r11, 0.0);
   if (r11 > 0.0) {
-    Ri[1] = make_double2(-r01.x / (r00 * r11), -r01.y / (r00 * r11));
-    Ri[3] = make_double2(1.0 / r11, 0.0);
+    const double i11 = 1.0 / r11, t = i00 * i11;
+    Ri[1] = make_double2(-r01.x * t, -r01.y * t);
+    Ri[3] = make_double2(i11, 0.0);
   }
   return bad;
 }
 
-__global__ void __launch_bounds__(32 * kRedLanes) sv_reduce_kernel(const __grid_constant__ SvReduceBatch batch) {
+__global__ void __launch_bounds__(kRedThreads) sv_reduce_kernel(const __grid_constant__ SvReduceBatch batch) {
   const SvReduceJob& J = batch.job[blockIdx.y];
-  const int cl = threadIdx.x & 31, k = threadIdx.x >> 5;
-  const int i = blockIdx.x * 32 + cl;
+  const int E = J.mode == 0 ? 8 : 4, lanes = kRedThreads / E;  // entries, chunks at a time
+  const int cl = threadIdx.x % E, k = threadIdx.x / E;
+  const int i = blockIdx.x * E + cl;
   const int nent = J.mode == 0 ? J.ncols * J.nb : J.nb * J.nb;
-  if (blockIdx.x * 32 >= nent) return;  // uniform over the block
+  if (blockIdx.x * E >= nent) return;  // uniform over the block
   double2 a0 = make_double2(0.0, 0.0), a1 = a0;
   if (i < nent) {
     int ch = k;
-    for (; ch + kRedLanes < J.nchunks; ch += 2 * kRedLanes) {
+    for (; ch + lanes < J.nchunks; ch += 2 * lanes) {
       const double2 v0 = J.part[(long long)ch * J.ldp + i];
-      const double2 v1 = J.part[(long long)(ch + kRedLanes) * J.ldp + i];
+      const double2 v1 = J.part[(long long)(ch + lanes) * J.ldp + i];
       a0.x += v0.x;
       a0.y += v0.y;
       a1.x += v1.x;
@@ -549,14 +711,19 @@ __global__ void __launch_bounds__(32 * kRedLanes) sv_reduce_kernel(const __grid_
       a0.y += v0.y;
     }
   }
-  __shared__ double2 red[kRedLanes][32];
+  __shared__ double2 red[kRedThreads / 32][8];
   __shared__ double2 fin[4];
-  red[k][cl] = make_double2(a0.x + a1.x, a0.y + a1.y);
+  a0 = make_double2(a0.x + a1.x, a0.y + a1.y);
+  for (int o = E; o < 32; o <<= 1) {
+    a0.x += __shfl_xor_sync(0xffffffffu, a0.x, o);
+    a0.y += __shfl_xor_sync(0xffffffffu, a0.y, o);
+  }
+  if ((threadIdx.x & 31) < E) red[threadIdx.x >> 5][cl] = a0;
   __syncthreads();
   if (k == 0 && i < nent) {
-    double2 s = make_double2(0.0, 0.0);
-#pragma unroll 8
-    for (int q = 0; q < kRedLanes; ++q) {
+    double2 s = red[0][cl];
+#pragma unroll
+    for (int q = 1; q < kRedThreads / 32; ++q) {
       s.x += red[q][cl].x;
       s.y += red[q][cl].y;
     }
@@ -603,6 +770,10 @@ __global__ void __launch_bounds__(32 * kRedLanes) sv_reduce_kernel(const __grid_
 }
 
 // ----------------------------------------------------------------- normalisation
+// the block times the inverse of its Cholesky factor, into the basis and into
+// the newest-vectors block, a thread per row; in the arithmetic of the new
+// vectors (six FP64 conversions and eight products per entry cost more than the
+// row's traffic on GB300's FP64 pipe)
 template <class Pol, int NB>
 __global__ void sv_normalize_kernel(const __grid_constant__ SvNormBatch batch, int N) {
   using T = typename Pol::T;
@@ -614,57 +785,57 @@ __global__ void sv_normalize_kernel(const __grid_constant__ SvNormBatch batch, i
   const Wt* w = static_cast<const Wt*>(J.w);
   for (long long row = (long long)blockIdx.x * blockDim.x + threadIdx.x; row < N;
        row += (long long)gridDim.x * blockDim.x) {
-    double2 v[NB];
+    typename Pol::S v[NB];
 #pragma unroll
-    for (int a = 0; a < NB; ++a) v[a] = Pol::wto_d(w[row * J.ldw + a]);
+    for (int a = 0; a < NB; ++a) v[a] = Pol::wload(w[row * J.ldw + a]);
 #pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      double re = 0.0, im = 0.0;
-#pragma unroll
-      for (int a = 0; a < NB; ++a) {
-        re += v[a].x * r[a * NB + b].x - v[a].y * r[a * NB + b].y;
-        im += v[a].x * r[a * NB + b].y + v[a].y * r[a * NB + b].x;
-      }
-      if (J.out_w) {
-        static_cast<Wt*>(J.dst1)[row * J.ld1 + b] = Pol::wfrom_d(make_double2(re, im));
-      } else {
-        T o;
-        o.x = (decltype(o.x))re;
-        o.y = (decltype(o.y))im;
-        static_cast<T*>(J.dst1)[row * J.ld1 + b] = o;
-        if (J.dst2) static_cast<T*>(J.dst2)[row * J.ld2 + b] = o;
-      }
+    for (int b = 0; b < NB; ++b) {  // column b of v R^-1 (upper triangular)
+      const T o = Pol::out(Pol::smul2(v[0], r[b], v[NB - 1], r[(NB - 1) * NB + b], b > 0));
+      static_cast<T*>(J.dst1)[row * J.ld1 + b] = o;
+      if (J.dst2) static_cast<T*>(J.dst2)[row * J.ld2 + b] = o;
     }
   }
 }
 
-// FUSE: the accurate pass (update + second Gram), else the FP32 second update
-template <class Pol, int NT, int NB, bool FUSE>
-void launch_update_nt(const SvBatch& b, int N, int rpc, int maxcols, cudaStream_t s) {
-  const int nchunks = (N + rpc - 1) / rpc;
-  if constexpr (!FUSE) {
-    const size_t smem = sizeof(double2) * (size_t)maxcols * NB;
-    if (smem > 48 * 1024)
-      SWI_CUDA_TRY(cudaFuncSetAttribute(sv_update_fast_kernel<Pol, NT, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)smem));
-    sv_update_fast_kernel<Pol, NT, NB><<<dim3(nchunks, b.n), kThreads, smem, s>>>(b, N, rpc);
-  } else {
-    const size_t smem = sizeof(double2) * ((size_t)maxcols * NB + (size_t)kWarps * NB * 32);
-    if (smem > 48 * 1024)
-      SWI_CUDA_TRY(cudaFuncSetAttribute(sv_update_kernel<Pol, NT, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)smem));
-    sv_update_kernel<Pol, NT, NB><<<dim3(nchunks, b.n), kThreads, smem, s>>>(b, N, rpc);
-  }
+template <class Pol, int RT, int NC2, int NB, int NBUF>
+void launch_update_rt(const SvBatch& b, int N, int rpc, int maxcols, cudaStream_t s) {
+  using ST = typename Pol::ST;
+  const size_t tile = sizeof(ST) * ((size_t)NB * 2 * maxcols + RT * NB * 2 + (size_t)NBUF * RT * Pol::ldt(maxcols));
+  // the row groups' sums share the space: (G - 1) NB cpad <= 224 NB entries of 16 bytes
+  const size_t smem = std::max(tile, sizeof(double2) * 224 * NB);
+  smem_opt_in(reinterpret_cast<const void*>(sv_update_kernel<Pol, RT, NC2, NB, NBUF>));
+  sv_update_kernel<Pol, RT, NC2, NB, NBUF><<<dim3((N + rpc - 1) / rpc, b.n), kThreads, smem, s>>>(b, N, rpc);
 }
 
-template <class Pol, int NB, bool FUSE>
+// rows per tile: three blocks of 256 threads share an SM's shared memory with two
+// tiles each (a complex128 tile of 32 rows up to 64 columns, 16 rows up to 128)
+template <class Pol, int NB>
 void launch_update(const SvBatch& b, int N, int rpc, int maxcols, cudaStream_t s) {
-  if (maxcols <= 64) launch_update_nt<Pol, 2, NB, FUSE>(b, N, rpc, maxcols, s);
-  else if (maxcols <= 128) launch_update_nt<Pol, 4, NB, FUSE>(b, N, rpc, maxcols, s);
-  else if (maxcols <= 256) launch_update_nt<Pol, 8, NB, FUSE>(b, N, rpc, maxcols, s);
-  else if (maxcols <= 384) launch_update_nt<Pol, 12, NB, FUSE>(b, N, rpc, maxcols, s);
-  else if (maxcols <= 512) launch_update_nt<Pol, 16, NB, FUSE>(b, N, rpc, maxcols, s);
-  else if constexpr (NB == 1) launch_update_nt<Pol, 32, NB, FUSE>(b, N, rpc, maxcols, s);
+  const int wide = sizeof(typename Pol::ST) == 8 ? 2 : 1;
+  if (maxcols <= 64 * wide) launch_update_rt<Pol, 32, 1, NB, 2>(b, N, rpc, maxcols, s);
+  else if (maxcols <= 128 * wide) launch_update_rt<Pol, 16, 1, NB, 2>(b, N, rpc, maxcols, s);
+  else if (maxcols <= 256) launch_update_rt<Pol, 8, 1, NB, 2>(b, N, rpc, maxcols, s);
+  else if (maxcols <= 512) launch_update_rt<Pol, 8, 2, NB, 2>(b, N, rpc, maxcols, s);
+  else if constexpr (NB == 1) launch_update_rt<Pol, 8, 4, NB, 1>(b, N, rpc, maxcols, s);
+  else throw Error{SWI_EINVAL, "Gram-Schmidt pass: at most 512 basis columns with 2-vector blocks"};
+}
+
+template <class Pol, int NB, int R>
+void launch_update_fast_r(const SvBatch& b, int N, int rpc, int maxcols, int stages, cudaStream_t s) {
+  const size_t smem = sizeof(typename Pol::ST) * (size_t)kWarps * stages * R * maxcols + sizeof(float2) * (size_t)maxcols * NB;
+  smem_opt_in(reinterpret_cast<const void*>(sv_update_fast_kernel<Pol, NB, R>));
+  sv_update_fast_kernel<Pol, NB, R><<<dim3((N + rpc - 1) / rpc, b.n), kThreads, smem, s>>>(b, N, rpc, stages);
+}
+
+// rows per warp: three blocks share an SM's shared memory up to 256 columns
+// (complex128); past 512 only one stage of one row fits a block
+template <class Pol, int NB>
+void launch_update_fast(const SvBatch& b, int N, int rpc, int maxcols, cudaStream_t s) {
+  const int wide = sizeof(typename Pol::ST) == 8 ? 2 : 1;
+  if (maxcols <= 64 * wide) launch_update_fast_r<Pol, NB, 4>(b, N, rpc, maxcols, 2, s);
+  else if (maxcols <= 128 * wide) launch_update_fast_r<Pol, NB, 2>(b, N, rpc, maxcols, 2, s);
+  else if (maxcols <= 512) launch_update_fast_r<Pol, NB, 1>(b, N, rpc, maxcols, 2, s);
+  else if constexpr (NB == 1) launch_update_fast_r<Pol, NB, 1>(b, N, rpc, maxcols, 1, s);
   else throw Error{SWI_EINVAL, "Gram-Schmidt pass: at most 512 basis columns with 2-vector blocks"};
 }
 
@@ -673,25 +844,27 @@ void launch_pass_nb(const SvBatch& b, int mode, int N, int rpc, int maxcols, cud
   const int nchunks = (N + rpc - 1) / rpc;
   if (mode == SV_GRAM) {
     const dim3 grid(nchunks, (maxcols + 31) / 32, b.n);
-    sv_gram_kernel<Pol, NB, true><<<grid, kThreads, 0, s>>>(b, N, rpc);
+    sv_gram_kernel<Pol, NB><<<grid, kThreads, 0, s>>>(b, N, rpc);
   } else if (mode == SV_UPDATE_GRAM) {
-    launch_update<Pol, NB, true>(b, N, rpc, maxcols, s);
+    launch_update<Pol, NB>(b, N, rpc, maxcols, s);
   } else if (mode == SV_UPDATE) {
-    launch_update<Pol, NB, false>(b, N, rpc, maxcols, s);
+    launch_update_fast<Pol, NB>(b, N, rpc, maxcols, s);
+  } else if (mode == SV_SCALE_WGRAM) {
+    sv_wgram_kernel<Pol, NB, true><<<dim3(nchunks, b.n), kThreads, 0, s>>>(b, N, rpc);
   } else {
-    sv_wgram_kernel<Pol, NB><<<dim3(nchunks, b.n), kThreads, 0, s>>>(b, N, rpc);
+    sv_wgram_kernel<Pol, NB, false><<<dim3(nchunks, b.n), kThreads, 0, s>>>(b, N, rpc);
   }
 }
 
 }  // namespace
 
 int sv_rows_per_chunk(int N, int njobs) {
-  // enough row chunks for about eight blocks per SM over the jobs, at most
-  // 1024 rows per chunk (the bound on the per-lane partial sums)
-  const long long target = 8LL * 152;
-  long long per = (long long)N * std::max(njobs, 1) / target;
-  per = std::max<long long>(256, std::min<long long>(1024, per));
-  return (int)((per + 7) / 8 * 8);
+  // one wave of the three blocks an SM holds, over the jobs; at least one tile of
+  // 32 rows (2,000 rows in four windows: 252 blocks; chunks of at least 256 rows
+  // left 32, each marching 32 rows per warp for ~110 us) and at most 1024 (the
+  // bound on the per-lane partial sums: several waves then)
+  const long long per = ((long long)N * std::max(njobs, 1) + 3 * 152 - 1) / (3 * 152);
+  return (int)std::max<long long>(32, std::min<long long>(1024, (per + 31) / 32 * 32));
 }
 
 void launch_sv_pass(const SvBatch& b, int mode, bool ds, int nb, int N, int rpc, cudaStream_t s,
@@ -701,7 +874,7 @@ void launch_sv_pass(const SvBatch& b, int mode, bool ds, int nb, int N, int rpc,
   int maxcols = 0;
   for (int q = 0; q < b.n; ++q) {
     const int nc = b.job[q].ncols;
-    if (nc > 1024 || (mode != SV_WGRAM && nc < 1))
+    if (nc > 1024 || (mode != SV_WGRAM && mode != SV_SCALE_WGRAM && nc < 1))
       throw Error{SWI_EINVAL, "Gram-Schmidt pass: 1..1024 basis columns"};
     maxcols = std::max(maxcols, nc);
   }
@@ -727,7 +900,7 @@ void launch_sv_reduce(const SvReduceBatch& b, cudaStream_t s, long long* launche
     if (J.mode == 2 && J.nb != 2) throw Error{SWI_EINVAL, "chunk reduction: second Cholesky pass needs nb = 2"};
     maxent = std::max(maxent, J.mode == 0 ? J.ncols * J.nb : J.nb * J.nb);
   }
-  sv_reduce_kernel<<<dim3((maxent + 31) / 32, b.n), 32 * kRedLanes, 0, s>>>(b);
+  sv_reduce_kernel<<<dim3((maxent + 7) / 8, b.n), kRedThreads, 0, s>>>(b);
   SWI_CHECK_LAUNCH();
   if (launches) ++*launches;
 }

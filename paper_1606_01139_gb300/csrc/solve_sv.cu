@@ -169,8 +169,9 @@ swi_status solve_sv(swi_ctx* c, const swi_solve_opts& opt, swi_solve_info* info)
     total_out += w.nreq;
   }
   // row chunks of the Gram-Schmidt passes: sized each step for the windows
-  // still expanding (at least 256 rows per chunk, so at most this many chunks)
-  const int max_chunks = (c->N + 255) / 256;
+  // still expanding; one window has the smallest chunks
+  const int min_rpc = swi::sv_rows_per_chunk(c->N, 1);
+  const int max_chunks = (c->N + min_rpc - 1) / min_rpc;
   for (int j = 0; j < nwin; ++j) {
     Win& w = *win[j];
     const size_t hh = (size_t)w.ldh * w.ldh;
@@ -233,40 +234,36 @@ swi_status solve_sv(swi_ctx* c, const swi_solve_opts& opt, swi_solve_info* info)
     }
   };
   // Orthonormalise the blocks W[:, j nb : j nb + nb] of the given windows:
-  // w^H w, one Cholesky factor for nb = 1, Cholesky-QR twice for nb = 2; R
-  // goes below the block's column of H (when hrow is set), the block into the
-  // basis at column dst_col and into Vcur.
-  auto orthonormalise = [&](const std::vector<Win*>& ws, const std::vector<int>& dst_col, bool hrow, int rpc) {
+  // w^H w (its partials already formed by the second update when have_gram),
+  // one Cholesky factor for nb = 1, Cholesky-QR twice for nb = 2; R goes below
+  // the block's column of H (when hrow is set), the block into the basis at
+  // column dst_col and into Vcur.
+  auto orthonormalise = [&](const std::vector<Win*>& ws, const std::vector<int>& dst_col, bool hrow, bool have_gram,
+                            int rpc) {
     const int na = (int)ws.size();
     const int nchunks = (c->N + rpc - 1) / rpc;
     swi::SvReduceBatch r1, r2;
-    swi::SvNormBatch n1, n2;
+    swi::SvNormBatch nm;
     swi::SvBatch g;
-    r1.n = r2.n = n1.n = n2.n = g.n = na;
+    r1.n = r2.n = nm.n = g.n = na;
     for (int q = 0; q < na; ++q) {
       Win& w = *ws[q];
       T* wc = Wblk.as<T>() + w.col * nb;
-      T* Qd = w.Q.template as<T>() + dst_col[q];
       double2* Hr = hrow ? w.H.template as<double2>() + (long long)(w.p + nb) * w.ldh + w.p : nullptr;
       double2* pp = w.part.template as<double2>();
       double2* ri = w.rinv.template as<double2>();
       r1.job[q] = swi::SvReduceJob{pp, w.ldh * nb, nchunks, 0, nb, 1, nullptr, nb == 1 ? Hr : nullptr, w.ldh, ri};
-      g.job[q] = swi::SvJob{w.Q.p, w.ldq, 0, wc, ldv, nullptr, pp, w.ldh * nb};
+      g.job[q] = swi::SvJob{w.Q.p, w.ldq, 0, wc, ldv, ri, pp, w.ldh * nb};
       r2.job[q] = swi::SvReduceJob{pp, w.ldh * nb, nchunks, 0, nb, 2, nullptr, Hr, w.ldh, ri};
-      if (nb == 1) {
-        n1.job[q] = swi::SvNormJob{wc, ldv, Qd, w.ldq, Vcur.as<T>() + w.col * nb, ldv, ri, 0};
-      } else {
-        n1.job[q] = swi::SvNormJob{wc, ldv, wc, ldv, nullptr, 0, ri, 1};
-        n2.job[q] = swi::SvNormJob{wc, ldv, Qd, w.ldq, Vcur.as<T>() + w.col * nb, ldv, ri, 0};
-      }
+      nm.job[q] = swi::SvNormJob{wc, ldv, w.Q.template as<T>() + dst_col[q], w.ldq, Vcur.as<T>() + w.col * nb, ldv, ri};
     }
-    swi::launch_sv_pass(g, swi::SV_WGRAM, DS, nb, c->N, rpc, c->stream, &c->launches);
+    if (!have_gram) swi::launch_sv_pass(g, swi::SV_WGRAM, DS, nb, c->N, rpc, c->stream, &c->launches);
     swi::launch_sv_reduce(r1, c->stream, &c->launches);
-    swi::launch_sv_normalize(n1, DS, nb, c->N, c->stream, &c->launches);
-    if (nb == 1) return;
-    swi::launch_sv_pass(g, swi::SV_WGRAM, DS, nb, c->N, rpc, c->stream, &c->launches);
-    swi::launch_sv_reduce(r2, c->stream, &c->launches);
-    swi::launch_sv_normalize(n2, DS, nb, c->N, c->stream, &c->launches);
+    if (nb == 2) {  // w R1^-1 and its Gram matrix in one pass
+      swi::launch_sv_pass(g, swi::SV_SCALE_WGRAM, DS, nb, c->N, rpc, c->stream, &c->launches);
+      swi::launch_sv_reduce(r2, c->stream, &c->launches);
+    }
+    swi::launch_sv_normalize(nm, DS, nb, c->N, c->stream, &c->launches);
   };
 
   // start blocks: random, orthonormalised, in columns [0, nb) of each basis and in Vcur
@@ -286,7 +283,7 @@ swi_status solve_sv(swi_ctx* c, const swi_solve_opts& opt, swi_solve_info* info)
         SWI_CHECK_LAUNCH();
       }
     }
-    orthonormalise(all, zero, false, swi::sv_rows_per_chunk(c->N, nwin));
+    orthonormalise(all, zero, false, false, swi::sv_rows_per_chunk(c->N, nwin));
   }
 
   const double tol_abs = rel_tol * anorm;
@@ -524,7 +521,7 @@ swi_status solve_sv(swi_ctx* c, const swi_solve_opts& opt, swi_solve_info* info)
     {
       ProfScope ps(c, SWI_K_CHOLQR, 8.0 * Nn * ncol * nb, sizeof(T) * Nn * ncol + 6.0 * wbytes);
       swi::launch_sv_pass(g2, swi::SV_UPDATE, DS, nb, c->N, rpc, c->stream, &c->launches);
-      orthonormalise(act, dst, true, rpc);
+      orthonormalise(act, dst, true, true, rpc);
     }
     // 3) windows whose next block would not fit: projected eigenproblem on their own stream
     for (int q = 0; q < na; ++q) {

@@ -320,7 +320,7 @@ void launch_sub_diag(double2* Y, int ldy, const double2* X, int ldx, const doubl
 // (complex64 in the FP32 form; in the double-single form four floats per
 // entry, the heads and tails of the real and imaginary parts), c the
 // [ncols][nb] FP64 coefficients, part [nchunks][ldp] FP64 chunk partials.
-enum { SV_GRAM = 0, SV_UPDATE_GRAM = 1, SV_UPDATE = 2, SV_WGRAM = 3 };
+enum { SV_GRAM = 0, SV_UPDATE_GRAM = 1, SV_UPDATE = 2, SV_WGRAM = 3, SV_SCALE_WGRAM = 4 };
 struct SvJob {
   const void* Q;
   int ldq, ncols;
@@ -335,13 +335,14 @@ struct SvBatch {
   SvJob job[kMaxBatch];
 };
 // SV_GRAM: part = Q^H w ([ncols][nb]); SV_UPDATE_GRAM: w -= Q c, then
-// part = Q^H w; SV_UPDATE: w -= Q c; SV_WGRAM: part = w^H w ([nb][nb], Q
-// unused).  ds: complex128 basis with double-single products (the Gram pass
+// part = Q^H w; SV_UPDATE: w -= Q c, then part = w^H w ([nb][nb]); SV_WGRAM:
+// part = w^H w (Q unused); SV_SCALE_WGRAM: w <- w c, c = R^-1 ([nb][nb]), then
+// part = w^H w.  ds: complex128 basis with double-single products (the Gram pass
 // and the update without a fused Gram in FP32, for the first pass and for the
 // second pass's small coefficients), else complex64 in FP32.
 void launch_sv_pass(const SvBatch& b, int mode, bool ds, int nb, int N, int rpc, cudaStream_t s,
                     long long* launches);
-// rows per chunk for njobs windows (256 to 1024, a multiple of 8)
+// rows per chunk for njobs windows (32 to 1024, a multiple of 32)
 int sv_rows_per_chunk(int N, int njobs);
 // Chunk sums.  mode 0: C[e] = sum of entry e < ncols * nb, added into
 // H[(e / nb) * ldh + e % nb] when H is set.  mode 1: the Gram matrix G = w^H w
@@ -363,9 +364,8 @@ struct SvReduceBatch {
   SvReduceJob job[kMaxBatch];
 };
 void launch_sv_reduce(const SvReduceBatch& b, cudaStream_t s, long long* launches);
-// dst1[:, b] (and dst2[:, b]) = sum_a w[:, a] r[a * nb + b] for b < nb, in the
-// basis element type (out_w = 0) or in w's own format (out_w = 1, dst2 unused;
-// in place allowed)
+// dst1[:, b] (and dst2[:, b]) = sum_a w[:, a] r[a * nb + b] for b < nb (r upper
+// triangular), in the basis element type
 struct SvNormJob {
   const void* w;
   int ldw;
@@ -374,7 +374,6 @@ struct SvNormJob {
   void* dst2;  // may be NULL
   int ld2;
   const double2* r;
-  int out_w;
 };
 struct SvNormBatch {
   int n;
