@@ -999,8 +999,6 @@ void ensure_RL(swi_ctx* c) {
   if (c->have_RL) return;
   const int n = c->npairs;
   const size_t nn = (size_t)n * n;
-  c->MR.ensure(sizeof(double2) * nn);
-  c->ML.ensure(sizeof(double2) * nn);
   c->Rm.ensure(sizeof(double2) * nn);
   c->Lm.ensure(sizeof(double2) * nn);
   c->Wm.ensure(sizeof(double2) * nn);
@@ -1018,8 +1016,19 @@ void ensure_RL(swi_ctx* c) {
     c->have_RL = true;
     return;
   }
-  gram_work_ensure(c, nn * 4);
   ProfScope ps(c, SWI_K_PROJ, 2.0 * 8.0 * c->N * (double)n * n, 2.0 * 16.0 * c->N * (double)n + 16.0 * c->N);
+  if (c->arith != SWI_ARITH_F64) {
+    const int chunks = swi::proj_ds_chunks(n, c->N);
+    gram_work_ensure(c, nn * 2 * (size_t)chunks);
+    swi::launch_proj_ds(c->U.as<double2>(), n, c->N, c->gR.as<double>(), c->gL.as<double>(),
+                        c->gram_work.as<double2>(), chunks, c->Rm.as<double2>(), c->Lm.as<double2>(),
+                        c->Wm.as<double2>(), c->stream, &c->launches);
+    c->have_RL = true;
+    return;
+  }
+  c->MR.ensure(sizeof(double2) * nn);
+  c->ML.ensure(sizeof(double2) * nn);
+  gram_work_ensure(c, nn * 4);
   swi::GramBatch gb;
   gb.n = 1;
   gb.job[0] = swi::GramJob{c->U.as<double2>(), c->U.as<double2>(), c->MR.as<double2>(), n, n, n, n, n, 0};
@@ -1620,21 +1629,33 @@ swi_status swi_grad(swi_ctx* c, int nE, const double* E, const double* dLdT, dou
       c->Mg.ensure(sizeof(double2) * (size_t)n * n);
       ProfScope ps(c, SWI_K_GRAD, 8.0 * (double)n * n * ((double)nE * n + c->N),
                    16.0 * c->N * (double)n * 2.0 + 8.0 * c->N);
-      swi::launch_gradM(c->Rm.as<double2>(), c->Lm.as<double2>(), c->eps.as<double2>(), n, c->Ebuf.as<double>(),
-                        c->wbuf.as<double>(), nE, c->Mg.as<double2>(), c->stream, &c->launches);
-      c->scratch.ensure(sizeof(double2) * (size_t)c->N * n);
-      swi::RowGemmBatch rb;
-      rb.n = 1;
-      rb.job[0] = swi::RowGemmJob{c->U.as<double2>(), c->Mg.as<double2>(), nullptr, c->scratch.as<double2>(), n, n, 0,
-                                  n, n, n, 1.0, 0.0};
-      rowgemm_dispatch(c->arith,rb, c->N, c->stream, &c->launches);
       DevMem tmp;
       double* dst = dLdV;
       if (!dLdV_on_device) {
         tmp.ensure(sizeof(double) * c->N);
         dst = tmp.as<double>();
       }
-      swi::launch_rowdot(c->scratch.as<double2>(), n, c->U.as<double2>(), n, n, c->N, dst, c->stream, &c->launches);
+      if (c->arith != SWI_ARITH_F64) {
+        const size_t nn = (size_t)n * n;
+        const int groups = swi::gradM_ds_groups(n, nE);
+        c->gsplit.ensure(sizeof(float4) * (2 * nn + (size_t)nE * n + 1));
+        gram_work_ensure(c, nn * (size_t)groups);
+        swi::launch_gradM_ds(c->Rm.as<double2>(), c->Lm.as<double2>(), c->eps.as<double2>(), n, c->Ebuf.as<double>(),
+                             c->wbuf.as<double>(), nE, groups, c->gsplit.as<float4>(), c->gram_work.as<double2>(),
+                             c->Mg.as<double2>(), c->stream, &c->launches);
+        swi::launch_rowquad_ds(c->U.as<double2>(), c->Mg.as<double2>(), n, c->N, c->gsplit.as<float4>(), dst,
+                               c->stream, &c->launches);
+      } else {
+        swi::launch_gradM(c->Rm.as<double2>(), c->Lm.as<double2>(), c->eps.as<double2>(), n, c->Ebuf.as<double>(),
+                          c->wbuf.as<double>(), nE, c->Mg.as<double2>(), c->stream, &c->launches);
+        c->scratch.ensure(sizeof(double2) * (size_t)c->N * n);
+        swi::RowGemmBatch rb;
+        rb.n = 1;
+        rb.job[0] = swi::RowGemmJob{c->U.as<double2>(), c->Mg.as<double2>(), nullptr, c->scratch.as<double2>(), n, n,
+                                    0, n, n, n, 1.0, 0.0};
+        rowgemm_dispatch(c->arith,rb, c->N, c->stream, &c->launches);
+        swi::launch_rowdot(c->scratch.as<double2>(), n, c->U.as<double2>(), n, n, c->N, dst, c->stream, &c->launches);
+      }
       if (!dLdV_on_device)
         SWI_CUDA_TRY(cudaMemcpyAsync(dLdV, dst, sizeof(double) * c->N, cudaMemcpyDeviceToHost, c->stream));
       sync(c->stream);

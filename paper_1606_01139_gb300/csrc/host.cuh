@@ -106,6 +106,7 @@ struct swi_ctx {
   int contract = SWI_CONTRACT_F64;
   bool have_RL = false;
   DevMem MR, ML, Rm, Lm, Wm, Mg, Ebuf, Tbuf, dEbuf, wbuf;
+  DevMem gsplit;                       // the adjoint's operands as pairs of floats
   DevMem R32, L32, part32, gt32, M32;  // FP32 contractions
   // workspaces
   DevMem gram_work, sig_dev, colwork, scratch, Uall, ordinfo, cholstat, ptrs, dres;
