@@ -4,10 +4,12 @@
 // work runs in FP32 and the accuracy comes from a subspace iteration:
 //
 //  1. mp_hess_kernel    Householder reduction of H to Hessenberg form, FP32
-//  2. mp_chase_kernel   QR iteration to Schur form, FP32, chains of up to 8
-//                       single-shift bulges three rows apart; the rotations go
-//                       to a list, the active block alone is updated
-//  3. mp_apply_kernel   Q = reflectors x rotations, a warp per four rows
+//  2. mp_chase_kernel   QR iteration to Schur form, FP32, chains of up to 16
+//                       single-shift bulges three rows apart until the blocks
+//                       that split off have order 32 or less, then a warp per
+//                       block; the rotations go to a list, the active block
+//                       alone is updated
+//  3. mp_apply_kernel   Q = reflectors x rotations, a warp per two rows
 //  4. mp_gemm (FP32)    T = Q^H H Q
 //  5. mp_order_kernel   the k kept Ritz values to the leading block, all
 //                       bubbles moving at once; its rotations applied to Q
@@ -25,7 +27,7 @@
 // thousand of them at order 150-208.  An FP32 chase step takes ~0.55 us and
 // moves all bulges of a chain (4-10 thousand steps), and the double-single chain
 // that remains has order k, a sixth to a half of m.  Measured per restart on one
-// GB300: 43 ms -> 6.5 ms at order 150 (15-35 kept), 57 ms -> 9.9 ms at orders
+// GB300: 43 ms -> 5.9 ms at order 150 (15-35 kept), 57 ms -> 9.6 ms at orders
 // 163-184 (35-110 kept); |H Z - Z T| / max|H| 0.6-2e-14, |Z^H Z - I| 2e-14 to
 // 2e-13 on restart matrices of orders 150-208.
 //
@@ -44,7 +46,8 @@ namespace swi {
 
 namespace {
 
-constexpr int kNB = 8;            // bulges per chain
+constexpr int kNB = 16;             // bulges per chain, rotations per list step
+constexpr int kSmall = 32;          // blocks up to this order are finished by a warp each
 constexpr int kChaseThreads = 32 * kNB;  // a warp per bulge
 constexpr int kMaxM = kMpMaxOrder;
 constexpr size_t kSmemMatrix = 220 * 1024;  // largest matrix kept in shared memory
@@ -359,6 +362,7 @@ struct Red {
   int ld, order;      // order < 0: ctl[CTL_K0]
   C *work, *Hp, *Vr;
   typename Arith<C>::R* tau;
+  int* len;           // rows of each reflector
   float4* rot;
   int max_steps, hmax_slot, steps_slot;
 };
@@ -391,14 +395,27 @@ __global__ void __launch_bounds__(THREADS, 1) mp_hess_kernel(const __grid_consta
   atomicMax(&s_hmax, __float_as_uint(hm));
   __syncthreads();
   for (int c = 0; c + 2 < m; ++c) {
-    const int nr = m - 1 - c;  // rows and columns c + 1 .. m - 1
-    // every warp forms the same reflector (no barrier for it)
+    // every warp forms the same reflector (no barrier for it); nr: rows and
+    // columns c + 1 .. c + nr, up to the column's last nonzero.  After a restart
+    // (a triangle, two coupling rows, a band) the support grows by two per
+    // column, so the first third of the columns is cheap
     R t2 = rzero(R{});
-    for (int i = 1 + lane; i < nr; i += 32) t2 = radd(t2, cnorm(A[(c + 1 + i) * m + c]));
+    int nr = 1;
+    for (int i = 1 + lane; i < m - 1 - c; i += 32) {
+      const C x = A[(c + 1 + i) * m + c];
+      if (abs1(x) > 0.f) nr = i + 1;
+      t2 = radd(t2, cnorm(x));
+    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t2 = radd(t2, rshx(t2, o));
+    for (int o = 16; o > 0; o >>= 1) {
+      t2 = radd(t2, rshx(t2, o));
+      nr = max(nr, __shfl_xor_sync(0xffffffffu, nr, o));
+    }
     if (!(hi(t2) > 1e-34f)) {
-      if (tid == 0) D.tau[c] = rzero(R{});
+      if (tid == 0) {
+        D.tau[c] = rzero(R{});
+        D.len[c] = 0;
+      }
       continue;
     }
     const C x0 = A[(c + 1) * m + c];
@@ -418,12 +435,16 @@ __global__ void __launch_bounds__(THREADS, 1) mp_hess_kernel(const __grid_consta
       v[i] = vi;
       D.Vr[(long long)c * m + c + 1 + i] = vi;
     }
-    if (tid == 0) D.tau[c] = tau;
+    if (tid == 0) {
+      D.tau[c] = tau;
+      D.len[c] = nr;
+    }
     __syncthreads();
-    const int ncp = (nr + 31) & ~31;
+    const int nc = m - 1 - c;  // columns of the left product
+    const int ncp = (nc + 31) & ~31;
     const int G = max(1, THREADS / ncp), g = tid / ncp, jj = tid - g * ncp;
     if (ncp <= THREADS) {
-      if (g < G && jj < nr) {
+      if (g < G && jj < nc) {
         C a0 = Arith<C>::zero(), a1 = a0;
         int i = g;
         for (; i + G < nr; i += 2 * G) {
@@ -434,7 +455,7 @@ __global__ void __launch_bounds__(THREADS, 1) mp_hess_kernel(const __grid_consta
         part[g * ncp + jj] = add(norm(a0), norm(a1));
       }
       __syncthreads();
-      for (int j = tid; j < nr; j += THREADS) {
+      for (int j = tid; j < nc; j += THREADS) {
         C s = part[j];
         for (int q = 1; q < G; ++q) s = add(s, part[q * ncp + j]);
         w[j] = scale(s, tau);
@@ -446,19 +467,19 @@ __global__ void __launch_bounds__(THREADS, 1) mp_hess_kernel(const __grid_consta
     for (int q = 0; q < NT; ++q) {
       const int j = lane + 32 * q;
       vr[q] = j < nr ? v[j] : Arith<C>::zero();
-      wr[q] = j < nr ? w[j] : Arith<C>::zero();
+      wr[q] = j < nc ? w[j] : Arith<C>::zero();
     }
     for (int i = warp; i < m; i += THREADS / 32) {
-      const bool below = i > c;
+      const bool below = i > c && i - c <= nr;
       C* Ar = A + i * m + c + 1 + lane;
       C row[NT], u = Arith<C>::zero();
 #pragma unroll
-      for (int q = 0; q < NT; ++q) row[q] = lane + 32 * q < nr ? Ar[32 * q] : Arith<C>::zero();
+      for (int q = 0; q < NT; ++q) row[q] = lane + 32 * q < (below ? nc : nr) ? Ar[32 * q] : Arith<C>::zero();
       if (below) {
         const C vi = cneg(v[i - c - 1]);
 #pragma unroll
         for (int q = 0; q < NT; ++q)
-          if (32 * q < nr) row[q] = fmadd(row[q], vi, wr[q]);
+          if (32 * q < nc) row[q] = fmadd(row[q], vi, wr[q]);
       }
 #pragma unroll
       for (int q = 0; q < NT; ++q)
@@ -466,7 +487,11 @@ __global__ void __launch_bounds__(THREADS, 1) mp_hess_kernel(const __grid_consta
       u = cneg(scale(lanes_sum(norm(u), 16), tau));
 #pragma unroll
       for (int q = 0; q < NT; ++q)
-        if (lane + 32 * q < nr) Ar[32 * q] = fmaddc(row[q], u, vr[q]);
+        if (32 * q < nr) {
+          if (lane + 32 * q < (below ? nc : nr)) Ar[32 * q] = fmaddc(row[q], u, vr[q]);
+        } else if (below && lane + 32 * q < nc) {
+          Ar[32 * q] = row[q];
+        }
       if (below && lane == 0) A[i * m + c] = i == c + 1 ? alpha : Arith<C>::zero();
     }
     __syncthreads();
@@ -490,23 +515,23 @@ __global__ void __launch_bounds__(THREADS, 1) mp_hess_kernel(const __grid_consta
 
 // ---------------------------------------------------------------- 2. the chase
 // eigenvalues of the trailing nb x nb block (approximate: a shift needs no
-// more), by one warp: at most two single-shift QR sweeps per eigenvalue on an
+// more), by one warp: at most one single-shift QR sweep per eigenvalue on an
 // FP32 copy in shared memory, lane j owning column j, then row j.  The copy is
 // taken relative to the last diagonal entry, so that the shift nearest it keeps
 // its full relative accuracy in the double-single form.
+__device__ __forceinline__ float2 wilkinson(float2 p, float2 q, float2 r, float2 d) {  // of [[p, q], [r, d]], nearer d
+  const float2 t = fc(0.5f * (p.x - d.x), 0.5f * (p.y - d.y)), bc = mulf(q, r);
+  float2 s2 = mulf(t, t);
+  s2 = sqrtf2(fc(s2.x + bc.x, s2.y + bc.y));
+  const float2 r1 = fc(t.x + s2.x, t.y + s2.y), r2 = fc(t.x - s2.x, t.y - s2.y);
+  const float2 den = norm2(r1) >= norm2(r2) ? r1 : r2;
+  if (!(norm2(den) > 0.f)) return d;
+  const float2 z = divf2(bc, den);
+  return fc(d.x - z.x, d.y - z.y);
+}
 template <class C>
 __device__ void chain_shifts(const C* H, int ihi, int nb, float2 (*a)[kNB + 1], float2* mu, bool exceptional) {
   const int lane = threadIdx.x & 31, o = ihi - nb + 1;
-  auto wilkinson = [](float2 p, float2 q, float2 r, float2 d) {  // of [[p, q], [r, d]], nearer d
-    const float2 t = fc(0.5f * (p.x - d.x), 0.5f * (p.y - d.y)), bc = mulf(q, r);
-    float2 s2 = mulf(t, t);
-    s2 = sqrtf2(fc(s2.x + bc.x, s2.y + bc.y));
-    const float2 r1 = fc(t.x + s2.x, t.y + s2.y), r2 = fc(t.x - s2.x, t.y - s2.y);
-    const float2 den = norm2(r1) >= norm2(r2) ? r1 : r2;
-    if (!(norm2(den) > 0.f)) return d;
-    const float2 z = divf2(bc, den);
-    return fc(d.x - z.x, d.y - z.y);
-  };
   const C last = H[offh(ihi) + ihi];
   if (nb == 1) {
     if (lane == 0)
@@ -520,8 +545,8 @@ __device__ void chain_shifts(const C* H, int ihi, int nb, float2 (*a)[kNB + 1], 
     }
     __syncwarp();
     for (int hi = nb - 1; hi > 0; --hi) {
-      for (int it = 0; it < 2; ++it) {
-        if (abs1(a[hi][hi - 1]) <= 1e-3f * (abs1(a[hi][hi]) + abs1(a[hi - 1][hi - 1]))) break;
+      for (int it = 0; it < 1; ++it) {
+        if (abs1(a[hi][hi - 1]) <= 1e-2f * (abs1(a[hi][hi]) + abs1(a[hi - 1][hi - 1]))) break;
         const float2 s = wilkinson(a[hi - 1][hi - 1], a[hi - 1][hi], a[hi][hi - 1], a[hi][hi]);
         for (int k = 0; k < hi; ++k) {
           const float2 x = k == 0 ? fc(a[0][0].x - s.x, a[0][0].y - s.y) : a[k][k - 1];
@@ -564,7 +589,8 @@ __global__ void __launch_bounds__(kChaseThreads, 1) mp_chase_kernel(const __grid
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ float2 s_mu[kNB];
   __shared__ float2 s_blk[kNB][kNB + 1];
-  __shared__ int s_l;
+  __shared__ int s_l, s_nblk, s_next, s_most, s_bad;
+  __shared__ short2 s_small[kMaxM / 2 + 1];
   if (ctl[CTL_STATUS] != 0) return;
   const int m = order_of(D.order, ctl), tid = threadIdx.x, lane = tid & 31, b = tid >> 5;
   C* H = SMEM ? reinterpret_cast<C*>(smem_raw) : D.Hp;
@@ -572,6 +598,7 @@ __global__ void __launch_bounds__(kChaseThreads, 1) mp_chase_kernel(const __grid
     for (int e = tid; e < offh(m); e += kChaseThreads) H[e] = D.Hp[e];
   const float hmax = __int_as_float(ctl[D.hmax_slot]);
   int ihi = m - 1, its = 0, sweeps = 0, step = 0, status = 0;
+  if (tid == 0) s_nblk = s_next = s_most = s_bad = 0;
   __syncthreads();
   while (ihi > 0) {
     // the largest index with a negligible subdiagonal
@@ -590,8 +617,15 @@ __global__ void __launch_bounds__(kChaseThreads, 1) mp_chase_kernel(const __grid
       its = 0;
       continue;
     }
+    if (ihi - l < kSmall) {  // left for the second phase
+      if (tid == 0) s_small[s_nblk++] = make_short2((short)l, (short)ihi);
+      __syncthreads();
+      ihi = l - 1;
+      its = 0;
+      continue;
+    }
     ++its;
-    const int nb = min(kNB, max(1, (ihi - l + 1) / 4));
+    const int nb = min(kNB, max(1, (ihi - l + 1) / 3));
     const int T = (ihi - l) + 3 * (nb - 1);
     if (++sweeps > 30 * m + 30 || step + T > D.max_steps) {
       status = 1;
@@ -616,6 +650,7 @@ __global__ void __launch_bounds__(kChaseThreads, 1) mp_chase_kernel(const __grid
           y = H[offh(k - 1) + k + 1];
         }
         g = make_rot(x, y, r);
+        __syncwarp();  // at the top of a block, x and y lie in the columns rotated next
         // columns k + lane, + 32, ... (two at a time: independent loads in flight);
         // offh(j + 32) - offh(j) = 32 j + 592
         int j = k + lane, at = offh(j) + k, step32 = 32 * j + 592;
@@ -670,6 +705,94 @@ __global__ void __launch_bounds__(kChaseThreads, 1) mp_chase_kernel(const __grid
       __syncthreads();
     }
   }
+  __syncthreads();
+  // ---- the small blocks, a warp each: single shifts, lane j owning a column of
+  // the row rotations, then a row of the column rotations.  A warp's rotations
+  // fill its own slot of the list from the last common step on; those of
+  // different blocks touch different columns.
+  const int nblk = s_nblk;
+  int mine = step;
+  if (status == 0) {
+    for (;;) {
+      int q = 0;
+      if (lane == 0) q = atomicAdd(&s_next, 1);
+      q = __shfl_sync(0xffffffffu, q, 0);
+      if (q >= nblk || s_bad) break;
+      const int l0 = s_small[q].x;
+      int top = s_small[q].y, it = 0, total = 0;
+      while (top > l0) {
+        // lane i tests the subdiagonal of row l0 + 1 + i
+        const int row = l0 + 1 + lane;
+        bool small = false;
+        if (row <= top) {
+          const float t = abs1(H[offh(row - 1) + row - 1]) + abs1(H[offh(row) + row]);
+          small = abs1(H[offh(row - 1) + row]) <= fmaxf(Defl<C>::rel * t, Defl<C>::abs * hmax);
+        }
+        const unsigned hit = __ballot_sync(0xffffffffu, small);
+        const int l = hit ? l0 + 32 - __clz(hit) : l0;
+        if (l == top) {
+          --top;
+          it = 0;
+          continue;
+        }
+        ++it;
+        if (++total > 40 * kSmall || mine + top - l > D.max_steps) {
+          s_bad = 1;
+          break;
+        }
+        const C last = H[offh(top) + top];
+        float2 mf = wilkinson(head(sub(H[offh(top - 1) + top - 1], last)), head(H[offh(top) + top - 1]),
+                              head(H[offh(top - 1) + top]), fc(0.f, 0.f));
+        if (it % 10 == 0) mf.x += 0.75f * abs1(H[offh(top - 1) + top]);
+        const C mu = plus_f(last, mf);
+        __syncwarp();
+        for (int k = l; k < top; ++k, ++mine) {
+          C x, y, r;
+          if (k == l) {
+            x = sub(H[offh(l) + l], mu);
+            y = H[offh(l) + l + 1];
+          } else {
+            x = H[offh(k - 1) + k];
+            y = H[offh(k - 1) + k + 1];
+          }
+          const RotT<C> g = make_rot(x, y, r);
+          __syncwarp();
+          const int j = k + lane;
+          if (j <= top) {
+            C* p = H + offh(j) + k;
+            C h0 = p[0], h1 = p[1];
+            rot_rows(h0, h1, g);
+            p[0] = h0;
+            p[1] = h1;
+          }
+          __syncwarp();
+          const int i = l + lane;
+          if (i <= min(k + 2, top)) {
+            C *p0 = H + offh(k), *p1 = p0 + k + 3;
+            C h0 = p0[i], h1 = p1[i];
+            rot_cols(h0, h1, g);
+            p0[i] = h0;
+            p1[i] = h1;
+          }
+          if (lane == 0) {
+            if (k > l) {
+              H[offh(k - 1) + k] = r;
+              H[offh(k - 1) + k + 1] = Arith<C>::zero();
+            }
+            put_rot(D.rot, (long long)mine * kNB + b, g, k);
+          }
+          __syncwarp();
+        }
+      }
+    }
+    if (lane == 0) atomicMax(&s_most, mine);
+  }
+  __syncthreads();
+  if (s_bad) status = 1;
+  if (status == 0) {
+    for (int q = mine + lane; q < s_most; q += 32) put_rot(D.rot, (long long)q * kNB + b, ident(C{}), -1);
+    step = s_most;
+  }
   if (tid == 0) {
     if (status) ctl[CTL_STATUS] = status;
     ctl[D.steps_slot] = status ? 0 : step;
@@ -678,10 +801,10 @@ __global__ void __launch_bounds__(kChaseThreads, 1) mp_chase_kernel(const __grid
 
 // ---------------------------------------------------------------- 3. rows x (reflectors, rotations)
 // Rows of Q (or of V) times the reflectors of a reduction (Vr set) and the
-// rotations of a list.  Four rows per warp in shared memory; a lane holds one
-// row and one of the (at most 8, disjoint) rotations of a step, so the steps of
+// rotations of a list.  Two rows per warp in shared memory; a lane holds one
+// row and one of the (at most 16, disjoint) rotations of a step, so the steps of
 // a warp need no barrier beyond its own.  src NULL: rows of the identity.
-constexpr int kApplyWarps = 2;
+constexpr int kApplyWarps = 4, kRows = 32 / kNB;  // rows per warp
 __device__ __forceinline__ double2 to_out(dc a) { return ds::cto(a); }
 __device__ __forceinline__ float2 to_out(float2 a) { return a; }
 __device__ __forceinline__ float2 load_row(const float2* p, float2) { return *p; }
@@ -693,10 +816,10 @@ __global__ void __launch_bounds__(32 * kApplyWarps)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (ctl[CTL_STATUS] != 0) return;
   const int m = order_of(D.order, ctl);
-  const int row = (blockIdx.x * kApplyWarps + warp) * 4 + (lane >> 3), b = lane & 7;
-  C* q = reinterpret_cast<C*>(smem_raw) + (size_t)(warp * 4 + (lane >> 3)) * (m + 1);
+  const int row = (blockIdx.x * kApplyWarps + warp) * kRows + lane / kNB, b = lane % kNB;
+  C* q = reinterpret_cast<C*>(smem_raw) + (size_t)(warp * kRows + lane / kNB) * (m + 1);
   const bool on = row < nrows;
-  for (int j = b; j < m; j += 8) {
+  for (int j = b; j < m; j += kNB) {
     C x = Arith<C>::zero();
     if (on && src) x = load_row(src + (long long)row * lds + j, C{});
     else if (on && j == row) set_one(x);
@@ -706,36 +829,41 @@ __global__ void __launch_bounds__(32 * kApplyWarps)
   if (reflect) {
     // all lanes on one row at a time, the reflector in registers (the next one
     // loaded meanwhile)
-    const C* q0 = reinterpret_cast<C*>(smem_raw) + (size_t)(warp * 4) * (m + 1);
+    C* q0 = reinterpret_cast<C*>(smem_raw) + (size_t)(warp * kRows) * (m + 1);
     C vn[NT];
     typename Arith<C>::R tn = D.tau[0];
+    int ln = D.len[0];
 #pragma unroll
-    for (int q = 0; q < NT; ++q) vn[q] = 1 + lane + 32 * q < m ? D.Vr[1 + lane + 32 * q] : Arith<C>::zero();
+    for (int q = 0; q < NT; ++q) vn[q] = lane + 32 * q < ln ? D.Vr[1 + lane + 32 * q] : Arith<C>::zero();
     for (int c = 0; c + 2 < m; ++c) {
       C v[NT];
       const typename Arith<C>::R tau = tn;
+      const int len = ln;
 #pragma unroll
       for (int q = 0; q < NT; ++q) v[q] = vn[q];
       if (c + 3 < m) {
         tn = D.tau[c + 1];
+        ln = D.len[c + 1];
         const C* src_v = D.Vr + (long long)(c + 1) * m + c + 2 + lane;
 #pragma unroll
-        for (int q = 0; q < NT; ++q) vn[q] = c + 2 + lane + 32 * q < m ? src_v[32 * q] : Arith<C>::zero();
+        for (int q = 0; q < NT; ++q) vn[q] = lane + 32 * q < ln ? src_v[32 * q] : Arith<C>::zero();
       }
       if (hi(tau) == 0.f) continue;
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        C* qr = const_cast<C*>(q0) + r * (m + 1) + c + 1 + lane;
+      for (int r = 0; r < kRows; ++r) {
+        C* qr = q0 + r * (m + 1) + c + 1 + lane;
         C x[NT], u = Arith<C>::zero();
 #pragma unroll
         for (int q = 0; q < NT; ++q) {
-          x[q] = c + 1 + lane + 32 * q < m ? qr[32 * q] : Arith<C>::zero();
-          fma2(u, x[q], v[q]);
+          if (32 * q < len) {
+            x[q] = lane + 32 * q < len ? qr[32 * q] : Arith<C>::zero();
+            fma2(u, x[q], v[q]);
+          }
         }
         u = cneg(scale(lanes_sum(norm(u), 16), tau));
 #pragma unroll
         for (int q = 0; q < NT; ++q)
-          if (c + 1 + lane + 32 * q < m) qr[32 * q] = fmaddc(x[q], u, v[q]);
+          if (lane + 32 * q < len) qr[32 * q] = fmaddc(x[q], u, v[q]);
       }
       __syncwarp();  // columns change lanes with c
     }
@@ -764,7 +892,7 @@ __global__ void __launch_bounds__(32 * kApplyWarps)
     }
   }
   if (on)
-    for (int j = b; j < m; j += 8) dst[(long long)row * lds + j] = to_out(q[j]);
+    for (int j = b; j < m; j += kNB) dst[(long long)row * lds + j] = to_out(q[j]);
 }
 
 // ---------------------------------------------------------------- 4./6. small products
@@ -1199,7 +1327,7 @@ __global__ void __launch_bounds__(512) mp_outcome_kernel(const __grid_constant__
     J.ordinfo[0] = k0;
     J.ordinfo[1] = s_n;
     J.ordinfo[2] = st != 0 ? 1 : 0;
-    J.ordinfo[3] = (int)(((long long)J.ctl[CTL_STEPSK] * kNB * 2 * k0) >> 10);  // Givens pair updates / 1024
+    J.ordinfo[3] = (int)(((long long)J.ctl[CTL_STEPSK] * 4 * 2 * k0) >> 10);  // Givens pair updates / 1024
   }
 }
 
@@ -1238,14 +1366,15 @@ size_t mp_schur_layout(MpJob* J, void* base, int m, int kcap, int ld, int b) {
   };
   const size_t mm = (size_t)m * m, mk = (size_t)m * kcap, kk = (size_t)kcap * kcap;
   MpJob t{};
-  t.max_steps = 80 * m + 2000;
+  t.max_steps = 60 * m + 2000;
   t.max_steps2 = (m + kNB - 1) / kNB * 2 * m;
-  t.max_stepsk = 80 * kcap + 2000;
+  t.max_stepsk = 60 * kcap + 2000;
   t.ctl = static_cast<int*>(take(64));
   t.H32 = static_cast<float2*>(take(8 * mm));
   t.Hp = static_cast<float2*>(take(8 * (size_t)offh(m)));
   t.Vr = static_cast<float2*>(take(8 * mm));
   t.tau = static_cast<float*>(take(4 * (size_t)m));
+  t.len = static_cast<int*>(take(4 * (size_t)m));
   t.Q = static_cast<float2*>(take(8 * mm));
   t.P = static_cast<float2*>(take(8 * mm));
   t.T = static_cast<float2*>(take(8 * (size_t)offu(m)));
@@ -1302,9 +1431,9 @@ void launch_schur_mp(const SchurJob& S, void* work, int kcap, cudaStream_t s, lo
     ++n;
   };
   auto tiles = [](int n_) { return (unsigned)((n_ + 15) / 16); };
-  auto rows8 = [](int n_) { return (unsigned)((n_ + 4 * kApplyWarps - 1) / (4 * kApplyWarps)); };
+  auto row_blocks = [](int n_) { return (unsigned)((n_ + kRows * kApplyWarps - 1) / (kRows * kApplyWarps)); };
   // ---- FP32 Schur form
-  const Red<float2> D{S.H, S.ld, m, J.H32, J.Hp, J.Vr, J.tau, J.rot, J.max_steps, CTL_HMAX, CTL_STEPS};
+  const Red<float2> D{S.H, S.ld, m, J.H32, J.Hp, J.Vr, J.tau, J.len, J.rot, J.max_steps, CTL_HMAX, CTL_STEPS};
   const size_t sq = 8 * (size_t)m * m;
   const int hs = sq <= kSmemMatrix - 28 * 1024 ? 1 : 0;  // beside the reflector, its product and partial sums
   auto hess = [&](auto kernel) {
@@ -1324,15 +1453,15 @@ void launch_schur_mp(const SchurJob& S, void* work, int kcap, cudaStream_t s, lo
   if (cs) chase(mp_chase_kernel<float2, true>, D, ph);
   else chase(mp_chase_kernel<float2, false>, D, 0);
   done();
-  const size_t qs = 8 * (size_t)kApplyWarps * 4 * (m + 1);
+  const size_t qs = 8 * (size_t)kApplyWarps * kRows * (m + 1);
   auto applyq = [&](const Red<float2>& P, const float2* src, int reflect) {
     auto go = [&](auto kernel) {
       allow_smem(kernel, qs);
-      kernel<<<rows8(m), 32 * kApplyWarps, qs, s>>>(P, J.ctl, m, src, J.Q, m, reflect);
+      kernel<<<row_blocks(m), 32 * kApplyWarps, qs, s>>>(P, J.ctl, m, src, J.Q, m, reflect);
     };
-    if (m <= 160) go(mp_apply_kernel<float2, float2, 8, 5>);
-    else if (m <= 256) go(mp_apply_kernel<float2, float2, 8, 8>);
-    else go(mp_apply_kernel<float2, float2, 8, 16>);
+    if (m <= 160) go(mp_apply_kernel<float2, float2, 16, 5>);
+    else if (m <= 256) go(mp_apply_kernel<float2, float2, 16, 8>);
+    else go(mp_apply_kernel<float2, float2, 16, 16>);
   };
   applyq(D, nullptr, 1);
   done();
@@ -1393,7 +1522,7 @@ void launch_schur_mp(const SchurJob& S, void* work, int kcap, cudaStream_t s, lo
   done();
   // ---- the double-single Schur form of the kept block, applied to V
   const Red<dc> K{J.G, S.ld, -1, static_cast<dc*>(J.Gd), static_cast<dc*>(J.Gp), static_cast<dc*>(J.Vk),
-                  static_cast<df*>(J.tauk), J.rotk, J.max_stepsk, CTL_HMAXK, CTL_STEPSK};
+                  static_cast<df*>(J.tauk), J.len, J.rotk, J.max_stepsk, CTL_HMAXK, CTL_STEPSK};
   const size_t kq = sizeof(dc) * (size_t)kcap * kcap;
   const int ks = kq <= kSmemMatrix - 44 * 1024 ? 1 : 0;
   auto hessk = [&](auto kernel) {
@@ -1409,14 +1538,14 @@ void launch_schur_mp(const SchurJob& S, void* work, int kcap, cudaStream_t s, lo
   if (kc) chase(mp_chase_kernel<dc, true>, K, kp);
   else chase(mp_chase_kernel<dc, false>, K, 0);
   done();
-  const size_t ks_rows = sizeof(dc) * (size_t)kApplyWarps * 4 * (kcap + 1);
+  const size_t ks_rows = sizeof(dc) * (size_t)kApplyWarps * kRows * (kcap + 1);
   auto applyk = [&](auto kernel) {
     allow_smem(kernel, ks_rows);
-    kernel<<<rows8(m), 32 * kApplyWarps, ks_rows, s>>>(K, J.ctl, m, J.V[cur], J.V[cur], kcap, 1);
+    kernel<<<row_blocks(m), 32 * kApplyWarps, ks_rows, s>>>(K, J.ctl, m, J.V[cur], J.V[cur], kcap, 1);
   };
-  if (kcap <= 96) applyk(mp_apply_kernel<dc, double2, 4, 3>);
-  else if (kcap <= 256) applyk(mp_apply_kernel<dc, double2, 4, 8>);
-  else applyk(mp_apply_kernel<dc, double2, 4, 16>);
+  if (kcap <= 96) applyk(mp_apply_kernel<dc, double2, 8, 3>);
+  else if (kcap <= 256) applyk(mp_apply_kernel<dc, double2, 8, 8>);
+  else applyk(mp_apply_kernel<dc, double2, 8, 16>);
   done();
   orth();
   project();

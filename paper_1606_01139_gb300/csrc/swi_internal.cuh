@@ -238,6 +238,7 @@ struct MpJob {
   int* ctl;                                                // control block (enum CTL_*)
   float2 *H32, *Hp, *Vr, *Q, *P, *T, *Tr, *R32, *X, *S32;       // FP32 work
   float* tau;
+  int* len;                                                // rows of each reflector
   float4 *rot, *rot2, *rotk;                               // rotation lists
   double2 *V[2], *W, *G, *BV;
   void *Gd, *Gp, *Vk, *tauk;                               // kept block in double-single
