@@ -1,13 +1,16 @@
 // Shifted stencil Y = (A - sigma_col) X on complex64 vectors with FP32
 // arithmetic (Eq. 1 applied matrix-free, shifted as in Eq. 3): the form for
-// blocks whose rows are not 16-byte aligned (an odd column count); the
-// TMA-staged kernel of stencil_c64_tma.cu serves the rest.  Each CTA owns a
-// 16 x 8 tile of (x, y) points and 4 columns and marches along z.  The 12
-// z-neighbours of a point live in a register queue (one new plane per step,
-// prefetched a step ahead); the x and y neighbours come from the current plane,
-// staged into shared memory with a 6-point cross-shaped halo (ghosts by odd
-// reflection or zero, as in the FP64 kernel), the next plane's staging loads
-// issued before this plane's arithmetic.  Layout: X, Y are [N][ld] complex64
+// blocks whose rows are not 16-byte aligned (an odd column count) and for grids
+// too small to fill the GPU with the deep tiles of stencil_c64_tma.cu.  A tile of
+// (x, y) points fitted to the grid (at most 512 points x columns) x 4 columns, or
+// 2 where no more are given, per CTA marches along z: the 13 z values of a point
+// in a register queue, the x and y neighbours from the current plane staged into
+// shared memory with a 6-point cross-shaped halo (ghosts by odd reflection or
+// zero), two buffers so that one barrier per plane suffices.  Latency bounds it,
+// so everything a plane needs is loaded two planes ahead and z is cut into whole
+// waves of CTAs.  Measured on one GB300: 45x37x91, 7 columns 26 us (fixed tiles of
+// 16 x 8 x 4 with a second wave of 28 CTAs took the same); 48x48x96, 2 columns ~20
+// us against 47 of the TMA-staged kernel.  Layout: X, Y are [N][ld] complex64
 // (float2), column index innermost.
 #include <algorithm>
 
@@ -17,9 +20,9 @@ namespace swi {
 
 namespace {
 
-constexpr int kTX = 16, kTY = 8, kNC = 4, kR = 6;
-constexpr int kThreadsC64 = kTX * kTY * kNC;
-constexpr int kSX = kTX + 2 * kR, kSY = kTY + 2 * kR;
+constexpr int kR = 6, kThreadsC64 = 512, kSlotsPerThread = 4;
+constexpr int kWave = 152;  // CTAs resident at once
+constexpr long long kMinTmaBlocks = 72;  // see launch_stencil_c64
 
 // value of column c at axis index j of a line whose in-range extent is n
 // (odd reflection about the planes -1 and n, or zero)
@@ -53,58 +56,54 @@ __device__ __forceinline__ float2 load_z(const float2* __restrict__ X, long long
   return make_float2(sgn * v.x, sgn * v.y);
 }
 
-// Staging slots of the cross-shaped halo: the kTY tile rows over the full
-// staged width, then the 2 kR halo rows over the tile's width; kNC columns each.
-constexpr int kSlotsA = kTY * kSX * kNC, kSlotsB = 2 * kR * kTX * kNC;
-constexpr int kSlots = kSlotsA + kSlotsB;
-constexpr int kSlotsPerThread = (kSlots + kThreadsC64 - 1) / kThreadsC64;
-
-template <int BC>
+template <int BC, int kNC>
 __global__ void __launch_bounds__(kThreadsC64, 1)
     stencil_c64_kernel(const __grid_constant__ StencilC64Params P, const float2* __restrict__ X, int ldx,
-                       float2* __restrict__ Y, int ldy, int ncols, const float* __restrict__ sigma, int zchunk) {
-  __shared__ float2 s[kSY][kSX][kNC];
-  const int cc = threadIdx.x % kNC;
-  const int tx = (threadIdx.x / kNC) % kTX;
-  const int ty = threadIdx.x / (kNC * kTX);
-  const int tiles_x = (P.nx + kTX - 1) / kTX;
-  const int x0 = (blockIdx.x % tiles_x) * kTX, y0 = (blockIdx.x / tiles_x) * kTY;
+                       float2* __restrict__ Y, int ldy, int ncols, const float* __restrict__ sigma, int zchunk, int TX,
+                       int TY) {
+  extern __shared__ float2 s_buf[];  // [2][TY + 12][TX + 12][kNC]
+  const int SX = TX + 2 * kR, SY = TY + 2 * kR;
+  const int cc = threadIdx.x % kNC, pt = threadIdx.x / kNC;
+  const int tx = pt % TX, ty = pt / TX;
+  const int tiles_x = (P.nx + TX - 1) / TX;
+  const int x0 = (blockIdx.x % tiles_x) * TX, y0 = (blockIdx.x / tiles_x) * TY;
   const int c0 = blockIdx.y * kNC;
   const int x = x0 + tx, y = y0 + ty, c = c0 + cc;
-  const bool mine = x < P.nx && y < P.ny && c < ncols;
+  const bool mine = pt < TX * TY && x < P.nx && y < P.ny && c < ncols;
   const int z0 = blockIdx.z * zchunk, z1 = min(P.nz, z0 + zchunk);
   const long long plane = (long long)P.nx * P.ny;
   const long long plane_ld = plane * ldx;
-  const long long pt_col = ((long long)y * P.nx + x) * ldx + c;
+  const long long prow = (long long)y * P.nx + x;  // point index within a plane
+  const long long pt_col = prow * ldx + c;
   float cm[kR + 1];
 #pragma unroll
   for (int m = 0; m <= kR; ++m) cm[m] = P.cm[m];
-  const float sig = mine ? sigma[c] : 0.f;
+  const float dcen = 3.f * cm[0] - (mine ? sigma[c] : 0.f);
 
-  // this thread's staging slots: smem index, source offset within a plane and
-  // sign (0: a zero ghost or an unused slot)
+  // staged cells of this thread: shared index, source offset within a plane and
+  // sign (0: a zero ghost or an unused cell)
   int soff[kSlotsPerThread], sidx[kSlotsPerThread];
   float ssg[kSlotsPerThread];
+  const int slots_a = TY * SX * kNC, slots = slots_a + 2 * kR * TX * kNC;
 #pragma unroll
   for (int k = 0; k < kSlotsPerThread; ++k) {
     const int e = threadIdx.x + k * kThreadsC64;
-    int sc, sx, sy;
-    if (e < kSlotsA) {
-      sc = e % kNC;
-      sx = (e / kNC) % kSX;
-      sy = kR + e / (kNC * kSX);
+    const int sc = e % kNC;
+    int sx, sy;
+    if (e < slots_a) {
+      sx = (e / kNC) % SX;
+      sy = kR + e / (kNC * SX);
     } else {
-      const int f = e - kSlotsA;
-      sc = f % kNC;
-      sx = kR + (f / kNC) % kTX;
-      const int r = f / (kNC * kTX);
-      sy = r < kR ? r : r + kTY;
+      const int f = (e - slots_a) / kNC;
+      sx = kR + f % TX;
+      const int r = f / TX;
+      sy = r < kR ? r : r + TY;
     }
     sidx[k] = -1;
     soff[k] = 0;
     ssg[k] = 0.f;
-    if (e < kSlots) {
-      sidx[k] = (sy * kSX + sx) * kNC + sc;
+    if (e < slots) {
+      sidx[k] = (sy * SX + sx) * kNC + sc;
       int srcx, srcy;
       float sgx, sgy;
       const int gc = c0 + sc;
@@ -114,72 +113,65 @@ __global__ void __launch_bounds__(kThreadsC64, 1)
       }
     }
   }
-  float2* sflat = &s[0][0][0];
+  const int buf = SX * SY * kNC;
+  const int here = ((kR + ty) * SX + kR + tx) * kNC + cc, row = SX * kNC;
 
   // z queue: q[k] = X at z - 6 + k, k = 0..12
   float2 q[2 * kR + 1];
 #pragma unroll
   for (int k = 0; k < 2 * kR + 1; ++k)
     q[k] = mine ? load_z<BC>(X, pt_col, plane_ld, z0 - kR + k, P.nz) : make_float2(0.f, 0.f);
-  const long long prow = (long long)y * P.nx + x;  // point index within a plane
-
-  // stage plane z0
-  float2 preA[kSlotsPerThread], preB[kSlotsPerThread];
-#pragma unroll
-  for (int k = 0; k < kSlotsPerThread; ++k)
-    preA[k] = ssg[k] != 0.f ? __ldg(X + (long long)z0 * plane_ld + soff[k]) : make_float2(0.f, 0.f);
-#pragma unroll
-  for (int k = 0; k < kSlotsPerThread; ++k)
-    if (sidx[k] >= 0) sflat[sidx[k]] = make_float2(ssg[k] * preA[k].x, ssg[k] * preA[k].y);
   // loads two steps ahead, alternating between the A and B register sets:
-  // staging values of plane z+1 / z+2, queue entries for planes z+7 / z+8,
-  // V and Gamma of planes z / z+1
-#pragma unroll
-  for (int k = 0; k < kSlotsPerThread; ++k)
-    preA[k] = (z0 + 1 < z1 && ssg[k] != 0.f) ? __ldg(X + (long long)(z0 + 1) * plane_ld + soff[k])
-                                             : make_float2(0.f, 0.f);
-  float2 nqA = mine ? load_z<BC>(X, pt_col, plane_ld, z0 + kR + 1, P.nz) : make_float2(0.f, 0.f), nqB;
-  float vA = mine ? __ldg(P.V + (long long)z0 * plane + prow) : 0.f, gA = mine ? __ldg(P.G + (long long)z0 * plane + prow) : 0.f;
-  float vB = 0.f, gB = 0.f;
-  __syncthreads();
-
-  auto step = [&](const int z, float2 (&pcur)[kSlotsPerThread], float2 (&pnxt)[kSlotsPerThread], float2& qcur,
-                  float2& qnxt, float& vcur, float& gcur, float& vnxt, float& gnxt) {
-    const bool more2 = z + 2 < z1;
+  // staging values of plane z + 1 / z + 2, queue entries for planes z + 7 / z + 8,
+  // V and Gamma of planes z / z + 1
+  float2 preA[kSlotsPerThread], preB[kSlotsPerThread];
+  const auto load_plane = [&](int z, float2 (&pre)[kSlotsPerThread]) {
+    const float2* Xz = X + (long long)z * plane_ld;
 #pragma unroll
     for (int k = 0; k < kSlotsPerThread; ++k)
-      pnxt[k] = (more2 && ssg[k] != 0.f) ? __ldg(X + (long long)(z + 2) * plane_ld + soff[k]) : make_float2(0.f, 0.f);
-    qnxt = mine ? load_z<BC>(X, pt_col, plane_ld, z + kR + 2, P.nz) : make_float2(0.f, 0.f);
+      pre[k] = (z < z1 && ssg[k] != 0.f) ? __ldg(Xz + soff[k]) : make_float2(0.f, 0.f);
+  };
+  const auto store_plane = [&](int z, const float2 (&pre)[kSlotsPerThread]) {
+    float2* nb = s_buf + ((z - z0) & 1) * buf;
+#pragma unroll
+    for (int k = 0; k < kSlotsPerThread; ++k)
+      if (sidx[k] >= 0) nb[sidx[k]] = make_float2(ssg[k] * pre[k].x, ssg[k] * pre[k].y);
+  };
+  load_plane(z0, preB);
+  load_plane(z0 + 1, preA);
+  float2 nqA = mine ? load_z<BC>(X, pt_col, plane_ld, z0 + kR + 1, P.nz) : make_float2(0.f, 0.f), nqB = nqA;
+  float vA = mine ? __ldg(P.V + (long long)z0 * plane + prow) : 0.f;
+  float gA = mine ? __ldg(P.G + (long long)z0 * plane + prow) : 0.f;
+  float vB = 0.f, gB = 0.f;
+  store_plane(z0, preB);
+  __syncthreads();
+
+  const auto step = [&](const int z, float2 (&pcur)[kSlotsPerThread], float2 (&pnxt)[kSlotsPerThread], float2& qcur,
+                        float2& qnxt, float& vcur, float& gcur, float& vnxt, float& gnxt) {
+    load_plane(z + 2, pnxt);
+    qnxt = mine && z + 2 < z1 ? load_z<BC>(X, pt_col, plane_ld, z + kR + 2, P.nz) : make_float2(0.f, 0.f);
     if (mine && z + 1 < z1) {
       vnxt = __ldg(P.V + (long long)(z + 1) * plane + prow);
       gnxt = __ldg(P.G + (long long)(z + 1) * plane + prow);
     }
     if (mine) {
-      const float d = 3.f * cm[0] + vcur - sig;
-      const float g = gcur;
-      const float2 x0v = q[kR];
-      float ar = fmaf(d, x0v.x, g * x0v.y);
-      float ai = fmaf(d, x0v.y, -g * x0v.x);
+      const float2* s = s_buf + ((z - z0) & 1) * buf + here;
+      const float d = dcen + vcur;
+      const float2 u = q[kR];
+      float2 a = make_float2(fmaf(d, u.x, gcur * u.y), fmaf(d, u.y, -gcur * u.x));
 #pragma unroll
       for (int m = 1; m <= kR; ++m) {
-        const float2 a = s[kR + ty][kR + tx - m][cc], b = s[kR + ty][kR + tx + m][cc];
-        const float2 u = s[kR + ty - m][kR + tx][cc], w = s[kR + ty + m][kR + tx][cc];
-        const float2 lo = q[kR - m], hi = q[kR + m];
-        ar = fmaf(cm[m], (a.x + b.x) + (u.x + w.x) + (lo.x + hi.x), ar);
-        ai = fmaf(cm[m], (a.y + b.y) + (u.y + w.y) + (lo.y + hi.y), ai);
+        const float2 t = __fadd2_rn(__fadd2_rn(__fadd2_rn(s[-m * kNC], s[m * kNC]), __fadd2_rn(s[-m * row], s[m * row])),
+                                    __fadd2_rn(q[kR - m], q[kR + m]));
+        a = __ffma2_rn(make_float2(cm[m], cm[m]), t, a);
       }
-      Y[((long long)z * plane + prow) * ldy + c] = make_float2(ar, ai);
+      Y[((long long)z * plane + prow) * ldy + c] = a;
     }
+    if (z + 1 < z1) store_plane(z + 1, pcur);
 #pragma unroll
     for (int k = 0; k < 2 * kR; ++k) q[k] = q[k + 1];
     q[2 * kR] = qcur;
-    __syncthreads();  // every read of plane z is done
-    if (z + 1 < z1) {
-#pragma unroll
-      for (int k = 0; k < kSlotsPerThread; ++k)
-        if (sidx[k] >= 0) sflat[sidx[k]] = make_float2(ssg[k] * pcur[k].x, ssg[k] * pcur[k].y);
-    }
-    __syncthreads();
+    __syncthreads();  // plane z + 1 is staged; plane z's buffer is written after the next barrier at the earliest
   };
   int z = z0;
   for (; z + 1 < z1; z += 2) {
@@ -189,27 +181,80 @@ __global__ void __launch_bounds__(kThreadsC64, 1)
   if (z < z1) step(z, preA, preB, nqA, nqB, vA, gA, vB, gB);
 }
 
+// Tile of at most 512 / kNC points: the extents that cover nx x ny with the
+// fewest CTAs and halo cells, each axis cut evenly
+void pick_tile(int nx, int ny, int kNC, int& TX, int& TY) {
+  double best = 1e300;
+  TX = TY = 8;
+  for (int t = std::min(8, nx); t <= std::min(nx, 64); ++t) {
+    const int u_max = std::min({ny, kThreadsC64 / kNC / t, 32});
+    const int bx = (nx + t - 1) / t, by = (ny + u_max - 1) / u_max;
+    const int w = (nx + bx - 1) / bx, v = (ny + by - 1) / by;
+    const int slots = (v * (w + 2 * kR) + 2 * kR * w) * kNC;
+    if (slots > kSlotsPerThread * kThreadsC64) continue;
+    // a CTA costs its full width of threads, and its halo
+    const double cost = (double)bx * by * (kThreadsC64 + 0.25 * slots);
+    if (cost < best) {
+      best = cost;
+      TX = w;
+      TY = v;
+    }
+  }
+}
+
+// Planes per CTA: a chunk of c planes costs about c + 2 plane times (filling the
+// queue), so the waves of resident CTAs times that is made small
+int pick_zchunk(long long ctas, int nz) {
+  int zchunk = nz;
+  double best = 1e300;
+  for (int n = 1; n <= nz; ++n) {
+    const int ch = (nz + n - 1) / n, m = (nz + ch - 1) / ch;
+    if (m != n) continue;
+    const double t = (double)((ctas * m + kWave - 1) / kWave) * (ch + 2);
+    if (t < best) {
+      best = t;
+      zchunk = ch;
+    }
+  }
+  return zchunk;
+}
+
 }  // namespace
 
 void launch_stencil_c64(const StencilC64Params& P, const float2* X, int ldx, float2* Y, int ldy, int ncols,
                         const float* sigma_dev, cudaStream_t s, long long* launches) {
   if (ncols <= 0) return;
-  if (P.VG != nullptr && stencil_c64_tma_ok(X, ldx)) {  // TMA-staged form (stencil_c64_tma.cu) for 16-byte aligned rows
+  // The TMA-staged kernel (16-byte aligned rows) has blocks of 32 x 8 points x 4
+  // columns x at least 24 planes: with few of them, or few of their columns in
+  // use, it leaves SMs or lanes idle.  Measured (this kernel / that one, us, each
+  // with ~40 of host time): 48x48x96 with 2 columns (48 blocks, half used) 53/83,
+  // with 8 (96) 78/80, with 16 (192) 112/88; 45x37x91 with 8 (60) 70/86; 64x64x128
+  // with 4 (80) 86/79, with 2 (80, half used) 65/81; 96x96x192 with 2 (288, half
+  // used) 112/109
+  const long long deep = (long long)((P.nx + 31) / 32) * ((P.ny + 7) / 8) * ((ncols + 3) / 4) * std::max(1, P.nz / 24);
+  if (deep * std::min(ncols, 4) >= kMinTmaBlocks * 4 && P.VG != nullptr && stencil_c64_tma_ok(X, ldx)) {
     launch_stencil_c64_tma(P, X, ldx, Y, ldy, ncols, sigma_dev, s, launches);
     return;
   }
-  const int tiles = ((P.nx + kTX - 1) / kTX) * ((P.ny + kTY - 1) / kTY);
+  int TX, TY;
+  const int kNC = ncols <= 2 ? 2 : 4;
+  pick_tile(P.nx, P.ny, kNC, TX, TY);
+  const int tiles = ((P.nx + TX - 1) / TX) * ((P.ny + TY - 1) / TY);
   const int cgroups = (ncols + kNC - 1) / kNC;
-  // z chunks: a CTA per SM or more, each chunk at least 16 planes deep so the
-  // 12-plane queue prologue stays a small fraction of the reads
-  int nzc = (152 + tiles * cgroups - 1) / (tiles * cgroups);
-  nzc = std::max(1, std::min(nzc, (P.nz + 15) / 16));
-  const int zchunk = (P.nz + nzc - 1) / nzc;
-  dim3 grid(tiles, cgroups, (P.nz + zchunk - 1) / zchunk);
-  if (P.bc == SWI_BC_ZERO)
-    stencil_c64_kernel<SWI_BC_ZERO><<<grid, kThreadsC64, 0, s>>>(P, X, ldx, Y, ldy, ncols, sigma_dev, zchunk);
-  else
-    stencil_c64_kernel<SWI_BC_ODD><<<grid, kThreadsC64, 0, s>>>(P, X, ldx, Y, ldy, ncols, sigma_dev, zchunk);
+  const int zchunk = pick_zchunk((long long)tiles * cgroups, P.nz);
+  const dim3 grid(tiles, cgroups, (P.nz + zchunk - 1) / zchunk);
+  // at most 42 KB: the slots of a tile bound its staged cells
+  const size_t smem = sizeof(float2) * 2 * (size_t)(TX + 2 * kR) * (TY + 2 * kR) * kNC;
+  auto go = [&](auto kernel) {
+    kernel<<<grid, kThreadsC64, smem, s>>>(P, X, ldx, Y, ldy, ncols, sigma_dev, zchunk, TX, TY);
+  };
+  if (kNC == 2) {
+    if (P.bc == SWI_BC_ZERO) go(stencil_c64_kernel<SWI_BC_ZERO, 2>);
+    else go(stencil_c64_kernel<SWI_BC_ODD, 2>);
+  } else {
+    if (P.bc == SWI_BC_ZERO) go(stencil_c64_kernel<SWI_BC_ZERO, 4>);
+    else go(stencil_c64_kernel<SWI_BC_ODD, 4>);
+  }
   SWI_CHECK_LAUNCH();
   if (launches) ++*launches;
 }
