@@ -18,9 +18,14 @@
 //    output receives its x and y terms and the diagonal, and output j - 6 is
 //    then complete and stored.  The sweep runs over planes z0 - 6 .. z1 + 5
 //    of the block's z range (ghost planes by reflection or zero);
-//  - each thread computes two points stacked in y for one column (the y
-//    neighbours of the pair come from one 14-value strip); the arithmetic is
-//    packed FP32x2 (re, im together).
+//  - each thread computes 2 x 2 points for one column: the x neighbours of a
+//    pair come from one 14-value strip, the y neighbours likewise, 13 reads of
+//    shared memory per output (shared-memory bandwidth bounds the kernel; with
+//    pairs in y alone it was 20).  Threads whose pair index has bit 1 set take
+//    their pair mirrored - the stencil is symmetric - so that the 64-byte steps
+//    of a quarter-warp fall on all 32 banks.  The arithmetic is packed FP32x2
+//    (re, im together).
+//    96x96x192, 16 columns on one GB300: 238 us against 257.
 // Ghost points: the tensor map fills out-of-range coordinates with zeros (the
 // zero rule, and the planes -1 and n of the odd rule); odd-reflection ghosts
 // further out are written into the staged box from their mirror points, and
@@ -41,7 +46,7 @@ namespace {
 constexpr int kTX = 32, kTY = 8, kR = 6, kNC = 4;
 constexpr int kBX = kTX + 2 * kR, kBY = kTY + 2 * kR;  // staged box (44 x 20 points)
 constexpr int kStages = 4;
-constexpr int kThreads = kTX * (kTY / 2) * kNC;  // 512: two points (y, y + 1) per thread
+constexpr int kThreads = (kTX / 2) * (kTY / 2) * kNC;  // 256: 2 x 2 points per thread
 constexpr int kBoxFloats = kBY * kBX * kNC * 2;    // 7040 floats = 28,160 bytes
 constexpr int kVGFloats = kTY * kTX * 2;           // (V, Gamma) of the tile: 2,048 bytes
 constexpr int kStageFloats = kBoxFloats + kVGFloats;  // 30,208 bytes (a multiple of 128)
@@ -132,23 +137,25 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ int s_nghost;
   const int tid = threadIdx.x;
   const int cc = tid % kNC;
-  const int px = (tid / kNC) % kTX;
-  const int py = tid / (kNC * kTX);
+  const int px = (tid / kNC) % (kTX / 2);
+  const int py = tid / (kNC * (kTX / 2));
+  const int dir = (px & 2) ? -1 : 1;                 // mirrored pairs: point 0 is the right one
+  const int bx0 = 2 * px + (dir < 0 ? 1 : 0);        // tile x of point 0; point 1 at bx0 + dir
   const int g = blockIdx.x % cgroups;
   const int tile = blockIdx.x / cgroups;
   const int x0 = (tile % tiles_x) * kTX, y0 = (tile / tiles_x) * kTY;
   const int c0 = g * kNC, c = c0 + cc;
   const int z0 = blockIdx.y * zchunk, z1 = min(P.nz, z0 + zchunk);
-  const int xa = x0 + px, ya = y0 + 2 * py;  // the pair's first point
+  const int xa = x0 + bx0, ya = y0 + 2 * py;  // the first point
   const long long plane = (long long)P.nx * P.ny;
   const bool colok = c < ncols;
-  bool ok[2];
-  long long pto[2];  // (point index within a plane) * ldy + c
+  bool ok[2][2];  // [dy][dx]
 #pragma unroll
-  for (int dy = 0; dy < 2; ++dy) {
-    ok[dy] = colok && xa < P.nx && ya + dy < P.ny;
-    pto[dy] = ((long long)(ya + dy) * P.nx + xa) * ldy + c;
-  }
+  for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
+    for (int dx = 0; dx < 2; ++dx) ok[dy][dx] = colok && xa + dx * dir < P.nx && ya + dy < P.ny;
+  const long long pt0 = ((long long)ya * P.nx + xa) * ldy + c;  // (point index within a plane) * ldy + c
+  const int ldx_pt = dir * ldy, ldy_pt = P.nx * ldy;
   float cm[kR + 1];
 #pragma unroll
   for (int m = 0; m <= kR; ++m) cm[m] = P.cm[m];
@@ -209,11 +216,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int t = 0; t < min(ns, kStages - 1); ++t) issue(t);
   }
 
-  float2 acc[2][kQ];  // pending outputs: plane js + t' in slot t' mod 13
+  float2 acc[4][kQ];  // pending outputs of point 2 dy + dx: plane js + t' in slot t' mod 13
 #pragma unroll
-  for (int dy = 0; dy < 2; ++dy)
+  for (int p = 0; p < 4; ++p)
 #pragma unroll
-    for (int k = 0; k < kQ; ++k) acc[dy][k] = make_float2(0.f, 0.f);
+    for (int k = 0; k < kQ; ++k) acc[p][k] = make_float2(0.f, 0.f);
 
   bool bad = false;
   int tlast = 0;
@@ -246,51 +253,62 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       float sg;
       src_plane(j, sg);
-      // the y strip of the pair (14 values); its entries 6 and 7 are the pair's own values
-      float2 sy[2 * kR + 2];
-      {
-        const float2* colp = S2 + ((2 * py) * kBX + px + kR) * kNC + cc;
+      // the y strips of the two columns of points (14 values each); entries 6 and 7 are the points' own
+      float2 sy[2][2 * kR + 2];
 #pragma unroll
-        for (int k = 0; k < 2 * kR + 2; ++k) sy[k] = colp[k * kBX * kNC];
+      for (int dx = 0; dx < 2; ++dx) {
+        const float2* colp = S2 + ((2 * py) * kBX + bx0 + dx * dir + kR) * kNC + cc;
+#pragma unroll
+        for (int k = 0; k < 2 * kR + 2; ++k) sy[dx][k] = colp[k * kBX * kNC];
       }
 #pragma unroll
-      for (int dy = 0; dy < 2; ++dy) {
-        const float2 uc = make_float2(sg * sy[dy + kR].x, sg * sy[dy + kR].y);
+      for (int p = 0; p < 4; ++p) {
+        const float2 v = sy[p & 1][(p >> 1) + kR];
+        const float2 uc = make_float2(sg * v.x, sg * v.y);
         // z terms: plane j into the pending outputs j - 6 .. j + 6 (not j itself)
 #pragma unroll
         for (int m = 1; m <= kR; ++m) {
           const float2 w = make_float2(cm[m], cm[m]);
-          acc[dy][(u + kQ - m) % kQ] = __ffma2_rn(w, uc, acc[dy][(u + kQ - m) % kQ]);
-          acc[dy][(u + m) % kQ] = __ffma2_rn(w, uc, acc[dy][(u + m) % kQ]);
+          acc[p][(u + kQ - m) % kQ] = __ffma2_rn(w, uc, acc[p][(u + kQ - m) % kQ]);
+          acc[p][(u + m) % kQ] = __ffma2_rn(w, uc, acc[p][(u + m) % kQ]);
         }
       }
       if (real) {
 #pragma unroll
         for (int dy = 0; dy < 2; ++dy) {
-          const float2 uc = sy[dy + kR];
-          const float2 vg = VG[(2 * py + dy) * kTX + px];
-          const float d = dcen + vg.x, gm = vg.y;
-          float2 a = acc[dy][u % kQ];
-          a.x += fmaf(d, uc.x, gm * uc.y);
-          a.y += fmaf(d, uc.y, -gm * uc.x);
-          // x neighbours (13 values of the point's row) and y neighbours (the strip)
-          const float2* row = S2 + ((2 * py + dy + kR) * kBX + px) * kNC + cc;
+          // the row's strip: values bx0 - 6 dir .. bx0 + 7 dir, the points' own at 6 and 7
+          const float2* row = S2 + ((2 * py + dy + kR) * kBX + bx0 + kR) * kNC + cc;
+          float2 sx[2 * kR + 2];
 #pragma unroll
-          for (int m = 1; m <= kR; ++m) {
-            const float2 t2 = f2add(f2add(row[(kR - m) * kNC], row[(kR + m) * kNC]),
-                                    f2add(sy[dy + kR - m], sy[dy + kR + m]));
-            a = __ffma2_rn(make_float2(cm[m], cm[m]), t2, a);
+          for (int k = 0; k < 2 * kR + 2; ++k)
+            sx[k] = (k == kR || k == kR + 1) ? sy[k - kR][dy + kR] : row[(k - kR) * dir * kNC];
+#pragma unroll
+          for (int dx = 0; dx < 2; ++dx) {
+            const int p = 2 * dy + dx;
+            const float2 uc = sy[dx][dy + kR];
+            const float2 vg = VG[(2 * py + dy) * kTX + bx0 + dx * dir];
+            const float d = dcen + vg.x, gm = vg.y;
+            float2 a = acc[p][u % kQ];
+            a.x += fmaf(d, uc.x, gm * uc.y);
+            a.y += fmaf(d, uc.y, -gm * uc.x);
+#pragma unroll
+            for (int m = 1; m <= kR; ++m) {
+              const float2 t2 = f2add(f2add(sx[dx + kR - m], sx[dx + kR + m]),
+                                      f2add(sy[dx][dy + kR - m], sy[dx][dy + kR + m]));
+              a = __ffma2_rn(make_float2(cm[m], cm[m]), t2, a);
+            }
+            acc[p][u % kQ] = a;
           }
-          acc[dy][u % kQ] = a;
         }
       }
       // output j - 6 is complete
       const int o = j - kR;
+      float2* yo = Y + (long long)o * plane * ldy + pt0;
 #pragma unroll
-      for (int dy = 0; dy < 2; ++dy) {
+      for (int p = 0; p < 4; ++p) {
         const int so = (u + kQ - kR) % kQ;
-        if (o >= z0 && ok[dy]) Y[(long long)o * plane * ldy + pto[dy]] = acc[dy][so];
-        acc[dy][so] = make_float2(0.f, 0.f);
+        if (o >= z0 && ok[p >> 1][p & 1]) yo[(long long)(p >> 1) * ldy_pt + (p & 1) * ldx_pt] = acc[p][so];
+        acc[p][so] = make_float2(0.f, 0.f);
       }
       __syncthreads();  // stage s is free for the copy issued next step
     }

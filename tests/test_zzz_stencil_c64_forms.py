@@ -29,6 +29,6 @@ def test_apply_c64(shape, nvec, bc):
         Y = c.apply_c64(X, sig)
     Xd = X.astype(np.complex128)
     sig32 = sig.astype(np.float32).astype(np.float64)
-    Yo = stencil.apply_A(Xd, w.nx, w.ny, w.nz, w.h, w.V, w.gamma_L, w.gamma_R, bc) - Xd * sig32[None, :]
+    Yo = stencil.apply_A(Xd, w.nx, w.ny, w.nz, w.h, w.V, w.gamma_L, w.gamma_R, bc=bc) - Xd * sig32[None, :]
     an = stencil.gershgorin_norm(w.h, w.V, w.gamma_L, w.gamma_R)
     assert np.max(np.abs(Y - Yo)) <= C64_TOL * an * np.max(np.abs(X))
