@@ -1607,7 +1607,7 @@ swi_status swi_grad(swi_ctx* c, int nE, const double* E, const double* dLdT, dou
     if (dLdV && c->contract == SWI_CONTRACT_F32) {
       copy_in(c->wbuf, dLdT, sizeof(double) * nE, false, c->stream);
       c->gt32.ensure(sizeof(float2) * (size_t)nE * n);
-      c->M32.ensure(sizeof(float2) * (size_t)n * n);
+      c->M32.ensure(sizeof(float2) * (size_t)n * n * 2);  // M and its symmetric part
       DevMem tmp;
       double* dst = dLdV;
       if (!dLdV_on_device) {
@@ -1618,8 +1618,8 @@ swi_status swi_grad(swi_ctx* c, int nE, const double* E, const double* dLdT, dou
         ProfScope ps(c, SWI_K_GRAD, 8.0 * (double)n * n * ((double)nE * n + c->N),
                      16.0 * c->N * (double)n + 8.0 * c->N);
         swi::launch_grad_f32(c->R32.as<float2>(), c->L32.as<float2>(), c->eps.as<double2>(), n, c->Ebuf.as<double>(),
-                             c->wbuf.as<double>(), nE, c->gt32.as<float2>(), c->M32.as<float2>(), c->U.as<double2>(),
-                             n, (long long)c->N, dst, c->stream, &c->launches);
+                             c->wbuf.as<double>(), nE, c->gt32.as<float2>(), c->M32.as<float2>(),
+                             c->M32.as<float2>() + (size_t)n * n, c->U.as<double2>(), n, (long long)c->N, dst, c->stream, &c->launches);
       }
       if (!dLdV_on_device)
         SWI_CUDA_TRY(cudaMemcpyAsync(dLdV, dst, sizeof(double) * c->N, cudaMemcpyDeviceToHost, c->stream));

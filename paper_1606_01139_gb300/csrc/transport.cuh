@@ -20,9 +20,9 @@ void launch_proj_f32(const double2* U, int ldu, int n, const double* gR, long lo
                      const double* gL, long long loL, long long hiL, float2* part, double2* R, double2* L,
                      double2* W, float2* R32, float2* L32, cudaStream_t s, long long* launches);
 // out[r] = 2 Re sum_ac U_ra M_ac U_rc with M = sum_e w_e D_e R conj(D_e) L^T D_e;
-// gt: nE x n complex64 scratch (the energy table), M: n x n complex64 scratch
+// gt: nE x n complex64 scratch (the energy table), M, S: n x n complex64 scratch
 void launch_grad_f32(const float2* R32, const float2* L32, const double2* eps, int n, const double* E,
-                     const double* w, int nE, float2* gt, float2* M, const double2* U, int ldu, long long N,
+                     const double* w, int nE, float2* gt, float2* M, float2* S, const double2* U, int ldu, long long N,
                      double* out, cudaStream_t s, long long* launches);
 // Double-single contractions (transport_ds.cu).  Projections: part holds
 // proj_ds_chunks(n, N) * 2 matrices of n x n complex128; writes R, L, W.

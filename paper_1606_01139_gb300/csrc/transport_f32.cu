@@ -18,8 +18,13 @@
 //    256 + (rows per chunk)/256 instead of the chunk length.
 //  - adjoint M: per energy, the tile of R conj(D_e) L^T over l, then scaled by
 //    w_e g_ea g_ec into the tile of M (the energy table g_e in FP32).
-//  - dL/dV: per 64-row block of U, (U M) tile by tile, each tile contracted
-//    with the same rows of U at once, so U M is never stored.
+//  - dL/dV as a symmetric form: per 64-row block of U, sum_{a <= c} S_ac U_ra
+//    tile by tile (S the sum of M and its transpose), each tile contracted with
+//    the same rows of U at once: half the products, nothing of size N x n stored.
+// FP32 issue bounds all three (4 x 4 complex outputs: 64 FMA per 8 shared loads).
+// Measured on one GB300, 1,000 pairs of 64x64x128, 256 energies: projections
+// 76 ms against 83, adjoint 114 against 167 (all of M, operands converted on
+// the FP64 pipe and loaded between barriers).
 #include <algorithm>
 #include <cfloat>
 
@@ -33,19 +38,40 @@ namespace {
 constexpr int kT = 64;    // output tile edge
 constexpr int kK = 16;    // contraction depth of one shared-memory stage
 constexpr int kThr = 256; // 16 x 16 threads, 4 x 4 outputs each (rows ty + 16 i, columns tx + 16 j)
-constexpr int kInner = 16;  // stages (of kK rows) summed before the block sum is added (projections)
+constexpr int kPer = kK * kT / kThr;  // staged entries of an operand per thread
+constexpr int kKP = 8;      // rows per stage of the projections
+constexpr int kInner = 32;  // stages (of kKP rows) summed before the block sum is added (projections)
 
-__device__ __forceinline__ float2 f2(double2 v) { return make_float2((float)v.x, (float)v.y); }
+// nearest float by integer arithmetic (a conversion instruction occupies the FP64
+// pipe, ~19 cycles of an SM per warp), without a branch, so that the loads of a
+// stage stay together; below 2^-126 zero, beyond the largest float infinity
+__device__ __forceinline__ float f1(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const unsigned top = (unsigned)(b >> 32), e = (top >> 20) & 0x7ff;
+  const unsigned m = ((unsigned)(b >> 29) & 0x7fffffu) | ((min(max(e, 897u), 1150u) - 896) << 23);
+  const unsigned low = (unsigned)b & 0x1fffffffu;
+  const unsigned r = m + (low + (m & 1u) > 0x10000000u);
+  const unsigned big = e == 0x7ff && (b << 12) != 0 ? 0x7fc00000u : 0x7f800000u;  // NaN stays NaN
+  return __uint_as_float((top & 0x80000000u) | (e < 897 ? 0u : (e > 1150 ? big : r)));
+}
+__device__ __forceinline__ float2 f2(double2 v) { return make_float2(f1(v.x), f1(v.y)); }
 __device__ __forceinline__ float2 f2zero() { return make_float2(0.f, 0.f); }
 // acc += a b
 __device__ __forceinline__ void fcfma(float2& acc, float2 a, float2 b) {
   acc.x = fmaf(a.x, b.x, fmaf(-a.y, b.y, acc.x));
   acc.y = fmaf(a.x, b.y, fmaf(a.y, b.x, acc.y));
 }
-// acc += conj(a) b
-__device__ __forceinline__ void fcfmac(float2& acc, float2 a, float2 b) {
-  acc.x = fmaf(a.x, b.x, fmaf(a.y, b.y, acc.x));
-  acc.y = fmaf(a.x, b.y, fmaf(-a.y, b.x, acc.y));
+// 4 x 4 outputs of a thread at one depth: 64 multiply-adds per 8 shared loads
+__device__ __forceinline__ void tile_step(float2 (&acc)[4][4], const float2* a, const float2* b) {
+  float2 xa[4], xb[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) xa[i] = a[16 * i];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) xb[j] = b[16 * j];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) fcfma(acc[i][j], xa[i], xb[j]);
 }
 __device__ __forceinline__ float2 fcmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
@@ -54,11 +80,11 @@ __device__ __forceinline__ float2 fcmul(float2 a, float2 b) {
 // part[s][a][c] = sum over the rows of chunk s of gamma_r conj(U_ra) U_rc, for
 // the upper tile pairs (ta <= tc): blockIdx.x enumerates them row by row of
 // tiles, blockIdx.y the chunks of rch rows of [lo, hi).
-__global__ void __launch_bounds__(kThr) proj_f32_kernel(const double2* __restrict__ U, int ldu, int n,
+__global__ void __launch_bounds__(kThr, 2) proj_f32_kernel(const double2* __restrict__ U, int ldu, int n,
                                                         const double* __restrict__ gam, long long lo, long long hi,
                                                         long long rch, int ntile, float2* __restrict__ part) {
-  __shared__ float2 sa[kK][kT];  // sa[k][col] = gamma_r U[r][a0 + col], r = row k of the stage
-  __shared__ float2 sc[kK][kT];  // sc[k][col] = U[r][c0 + col]
+  __shared__ float2 sa[kKP][kT];  // sa[k][col] = conj(gamma_r U[r][a0 + col]), r = row k of the stage
+  __shared__ float2 sc[kKP][kT];  // sc[k][col] = U[r][c0 + col]
   int t = blockIdx.x, ta = 0;
   while (t >= ntile - ta) {
     t -= ntile - ta;
@@ -75,36 +101,32 @@ __global__ void __launch_bounds__(kThr) proj_f32_kernel(const double2* __restric
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[i][j] = tot[i][j] = f2zero();
   int stage = 0;
-  for (long long r0 = rb; r0 < re; r0 += kK) {
-    for (int q = threadIdx.x; q < kK * kT; q += kThr) {
-      const int k = q / kT, col = q % kT;  // column fastest: coalesced rows of U
+  constexpr int kPerP = kKP * kT / kThr;
+  double2 pa[kPerP], pc[kPerP];  // the next stage, in flight during this one's products
+  const auto fetch = [&](long long r0) {
+#pragma unroll
+    for (int u = 0; u < kPerP; ++u) {
+      const int q = threadIdx.x + u * kThr, k = q / kT, col = q % kT;  // column fastest: coalesced rows of U
       const long long r = r0 + k;
-      float2 va = f2zero(), vc = f2zero();
-      if (r < re) {
-        const double2* Ur = U + r * (long long)ldu;
-        if (a0 + col < n) {
-          const float g = (float)gam[r];
-          const float2 u = f2(Ur[a0 + col]);
-          va = make_float2(g * u.x, g * u.y);
-        }
-        if (c0 + col < n) vc = f2(Ur[c0 + col]);
-      }
-      sa[k][col] = va;
-      sc[k][col] = vc;
+      const double2* Ur = U + r * (long long)ldu;
+      pa[u] = r < re && a0 + col < n ? __ldg(Ur + a0 + col) : make_double2(0.0, 0.0);
+      pc[u] = r < re && c0 + col < n ? __ldg(Ur + c0 + col) : make_double2(0.0, 0.0);
     }
+  };
+  fetch(rb);
+  for (long long r0 = rb; r0 < re; r0 += kKP) {
+#pragma unroll
+    for (int u = 0; u < kPerP; ++u) {
+      const int q = threadIdx.x + u * kThr, k = q / kT, col = q % kT;
+      const float g = r0 + k < re ? f1(__ldg(gam + r0 + k)) : 0.f;
+      const float2 v = f2(pa[u]);
+      sa[k][col] = make_float2(g * v.x, -g * v.y);
+      sc[k][col] = f2(pc[u]);
+    }
+    if (r0 + kKP < re) fetch(r0 + kKP);
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < kK; ++k) {
-      float2 xa[4], xc[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) xa[i] = sa[k][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) xc[j] = sc[k][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) fcfmac(acc[i][j], xa[i], xc[j]);
-    }
+    for (int k = 0; k < kKP; ++k) tile_step(acc, &sa[k][ty], &sc[k][tx]);
     __syncthreads();
     if (++stage == kInner) {
       stage = 0;
@@ -206,17 +228,7 @@ __global__ void __launch_bounds__(kThr) gradM_f32_kernel(const float2* __restric
       }
       __syncthreads();
 #pragma unroll
-      for (int ll = 0; ll < kK; ++ll) {
-        float2 xr[4], xl[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) xr[i] = sr[ll][ty + 16 * i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) xl[j] = sl[ll][tx + 16 * j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) fcfma(acc[i][j], xr[i], xl[j]);
-      }
+      for (int ll = 0; ll < kK; ++ll) tile_step(acc, &sr[ll][ty], &sl[ll][tx]);
       __syncthreads();
     }
 #pragma unroll
@@ -245,12 +257,28 @@ __global__ void __launch_bounds__(kThr) gradM_f32_kernel(const float2* __restric
   }
 }
 
-// out[r] = 2 Re sum_{a,c} U_ra M_ac U_rc for the 64 rows r0 .. r0 + 63 of a block
-__global__ void __launch_bounds__(kThr) rowquad_f32_kernel(const double2* __restrict__ U, int ldu,
-                                                           const float2* __restrict__ M, int n, long long N,
-                                                           double* __restrict__ out) {
+// S[a][c] = M_ac + M_ca for a < c, M_aa, zero below the diagonal: the quadratic
+// form needs no more, and half the products
+__global__ void symm_kernel(const float2* __restrict__ M, int n, float2* __restrict__ S) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (long long)n * n) return;
+  const int a = (int)(t / n), c = (int)(t % n);
+  float2 v = f2zero();
+  if (a <= c) v = M[t];
+  if (a < c) {
+    const float2 w = M[(size_t)c * n + a];
+    v = make_float2(v.x + w.x, v.y + w.y);
+  }
+  S[t] = v;
+}
+
+// out[r] = 2 Re sum_c U_rc sum_{a <= c} S_ac U_ra for the 64 rows r0 .. r0 + 63 of
+// a block; a stage's operands are loaded during the products of the one before
+__global__ void __launch_bounds__(kThr, 2) rowquad_f32_kernel(const double2* __restrict__ U, int ldu,
+                                                              const float2* __restrict__ S, int n, long long N,
+                                                              double* __restrict__ out) {
   __shared__ float2 su[kK][kT + 1];  // su[a][row] = U[r0 + row][a0 + a]
-  __shared__ float2 sm[kK][kT];      // sm[a][col] = M[a0 + a][c0 + col]
+  __shared__ float2 sm[kK][kT];      // sm[a][col] = S[a0 + a][c0 + col]
   const long long r0 = (long long)blockIdx.x * kT;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   float prow[4] = {0.f, 0.f, 0.f, 0.f};
@@ -260,36 +288,41 @@ __global__ void __launch_bounds__(kThr) rowquad_f32_kernel(const double2* __rest
     for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j) acc[i][j] = f2zero();
-    for (int a0 = 0; a0 < n; a0 += kK) {
-      for (int q = threadIdx.x; q < kK * kT; q += kThr) {
+    const int a1 = min(n, c0 + kT);
+    double2 pu[kPer];
+    float2 pm[kPer];
+    const auto fetch = [&](int a0) {
+#pragma unroll
+      for (int u = 0; u < kPer; ++u) {
+        const int q = threadIdx.x + u * kThr;
         {
           const int aa = q % kK, row = q / kK;  // 16 consecutive columns of one row of U
           const long long r = r0 + row;
           const int a = a0 + aa;
-          su[aa][row] = (r < N && a < n) ? f2(U[r * ldu + a]) : f2zero();
+          pu[u] = (r < N && a < n) ? __ldg(U + r * ldu + a) : make_double2(0.0, 0.0);
         }
         {
-          const int col = q % kT, ab = q / kT;  // 64 consecutive columns of one row of M
+          const int col = q % kT, ab = q / kT;  // 64 consecutive columns of one row of S
           const int a = a0 + ab, c = c0 + col;
-          sm[ab][col] = (a < n && c < n) ? M[(size_t)a * n + c] : f2zero();
+          pm[u] = (a < n && c < n) ? __ldg(S + (size_t)a * n + c) : f2zero();
         }
       }
+    };
+    fetch(0);
+    for (int a0 = 0; a0 < a1; a0 += kK) {
+#pragma unroll
+      for (int u = 0; u < kPer; ++u) {
+        const int q = threadIdx.x + u * kThr;
+        su[q % kK][q / kK] = f2(pu[u]);
+        sm[q / kT][q % kT] = pm[u];
+      }
+      if (a0 + kK < a1) fetch(a0 + kK);
       __syncthreads();
 #pragma unroll
-      for (int aa = 0; aa < kK; ++aa) {
-        float2 xu[4], xm[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) xu[i] = su[aa][ty + 16 * i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) xm[j] = sm[aa][tx + 16 * j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) fcfma(acc[i][j], xu[i], xm[j]);
-      }
+      for (int aa = 0; aa < kK; ++aa) tile_step(acc, &su[aa][ty], &sm[aa][tx]);
       __syncthreads();
     }
-    // contract the tile of U M with U[r][c0 + col] at once
+    // contract the tile with U[r][c0 + col] at once
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const long long r = r0 + ty + 16 * i;
@@ -368,8 +401,8 @@ void launch_proj_f32(const double2* U, int ldu, int n, const double* gR, long lo
 }
 
 void launch_grad_f32(const float2* R32, const float2* L32, const double2* eps, int n, const double* E,
-                     const double* w, int nE, float2* gt, float2* M, const double2* U, int ldu, long long N,
-                     double* out, cudaStream_t s, long long* launches) {
+                     const double* w, int nE, float2* gt, float2* M, float2* S, const double2* U, int ldu,
+                     long long N, double* out, cudaStream_t s, long long* launches) {
   if (n <= 0 || N <= 0) return;
   const long long ne = (long long)nE * n;
   if (ne > 0) {
@@ -381,9 +414,12 @@ void launch_grad_f32(const float2* R32, const float2* L32, const double2* eps, i
   gradM_f32_kernel<<<dim3(nt, nt), kThr, 0, s>>>(R32, L32, gt, w, n, nE, M);
   SWI_CHECK_LAUNCH();
   if (launches) ++*launches;
-  rowquad_f32_kernel<<<(unsigned)((N + kT - 1) / kT), kThr, 0, s>>>(U, ldu, M, n, N, out);
+  const long long nn = (long long)n * n;
+  symm_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(M, n, S);
   SWI_CHECK_LAUNCH();
-  if (launches) ++*launches;
+  rowquad_f32_kernel<<<(unsigned)((N + kT - 1) / kT), kThr, 0, s>>>(U, ldu, S, n, N, out);
+  SWI_CHECK_LAUNCH();
+  if (launches) *launches += 2;
 }
 
 }  // namespace swi
