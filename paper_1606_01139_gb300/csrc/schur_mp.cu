@@ -25,7 +25,7 @@
 // The chain of dependent rotations is what bounds the whole step: the order-m
 // double-single kernel (schur_ds.cu, one CTA) takes ~1.9 us per rotation, 17-38
 // thousand of them at order 150-208.  An FP32 chase step takes ~0.55 us and
-// moves all bulges of a chain (4-10 thousand steps), and the double-single chain
+// moves all bulges of a chain (3-7 thousand steps), and the double-single chain
 // that remains has order k, a sixth to a half of m.  Measured per restart on one
 // GB300: 43 ms -> 5.9 ms at order 150 (15-35 kept), 57 ms -> 9.6 ms at orders
 // 163-184 (35-110 kept); |H Z - Z T| / max|H| 0.6-2e-14, |Z^H Z - I| 2e-14 to
