@@ -1017,15 +1017,6 @@ void ensure_RL(swi_ctx* c) {
     return;
   }
   ProfScope ps(c, SWI_K_PROJ, 2.0 * 8.0 * c->N * (double)n * n, 2.0 * 16.0 * c->N * (double)n + 16.0 * c->N);
-  if (c->arith != SWI_ARITH_F64) {
-    const int chunks = swi::proj_ds_chunks(n, c->N);
-    gram_work_ensure(c, nn * 2 * (size_t)chunks);
-    swi::launch_proj_ds(c->U.as<double2>(), n, c->N, c->gR.as<double>(), c->gL.as<double>(),
-                        c->gram_work.as<double2>(), chunks, c->Rm.as<double2>(), c->Lm.as<double2>(),
-                        c->Wm.as<double2>(), c->stream, &c->launches);
-    c->have_RL = true;
-    return;
-  }
   c->MR.ensure(sizeof(double2) * nn);
   c->ML.ensure(sizeof(double2) * nn);
   gram_work_ensure(c, nn * 4);

@@ -24,11 +24,7 @@ void launch_proj_f32(const double2* U, int ldu, int n, const double* gR, long lo
 void launch_grad_f32(const float2* R32, const float2* L32, const double2* eps, int n, const double* E,
                      const double* w, int nE, float2* gt, float2* M, float2* S, const double2* U, int ldu, long long N,
                      double* out, cudaStream_t s, long long* launches);
-// Double-single contractions (transport_ds.cu).  Projections: part holds
-// proj_ds_chunks(n, N) * 2 matrices of n x n complex128; writes R, L, W.
-int proj_ds_chunks(int n, long long N);
-void launch_proj_ds(const double2* U, int n, long long N, const double* gR, const double* gL, double2* part,
-                    int chunks, double2* R, double2* L, double2* W, cudaStream_t s, long long* launches);
+// Double-single contractions of the adjoint (transport_ds.cu).
 // M = sum_e w_e D_e R conj(D_e) L^T D_e; split: 2 n^2 + nE n entries of scratch,
 // part: gradM_ds_groups(n, nE) matrices of n x n
 int gradM_ds_groups(int n, int nE);

@@ -1,7 +1,6 @@
-// The dense contractions of T(E) and its adjoint in double-single arithmetic on
+// The dense contractions of the adjoint of T(E) in double-single arithmetic on
 // the FP32 pipes (the FP64-class form):
 //
-//   M_R = U^H Gamma_R U, M_L = U^H Gamma_L U   (Hermitian: the upper tiles)
 //   M[a][c] = sum_e w_e g_ea g_ec sum_l R[a][l] conj(g_el) L[c][l]
 //   dL/dV(r) = 2 Re sum_ac U_ra M_ac U_rc = 2 Re sum_c U_rc sum_{a <= c} S_ac U_ra,
 //              S_ac = M_ac + M_ca (a < c), S_aa = M_aa
@@ -10,15 +9,13 @@
 // product exact up to its tail, heads summed by TwoSum), so a thread holds
 // several outputs, real and imaginary parts go through packed FP32x2
 // instructions (half the issue slots; the rest carry loads and splits), and
-// nothing inside the loops touches the FP64 pipe.  Both projections share one
-// pass over U.  Sums run in double-single over at most 1,024 terms and in FP64
-// beyond.
+// nothing inside the loops touches the FP64 pipe.  Sums run in double-single over
+// at most 1,024 terms and in FP64 beyond.
 //
 // Measured on one GB300, 400 pairs of the 48x48x96 grid, 128 energies:
-// projections 59 ms against 149 (one product at a time, all tiles, one absorber
-// after the other); adjoint 49 ms against 176 (M in native FP64, ~119; U M as an
-// N x n product, then a row dot: all of M, and 1.4 GB of scratch).  48 pairs of
-// the 10x10x20 grid, 32 energies: adjoint 0.10 ms against 2.7.
+// adjoint 49 ms against 176 (M in native FP64, ~119; U M as an N x n product, then
+// a row dot: all of M, and 1.4 GB of scratch).  48 pairs of the 10x10x20 grid, 32
+// energies: 0.10 ms against 2.7.
 #include <algorithm>
 
 #include "ds.cuh"
@@ -80,139 +77,6 @@ __device__ __forceinline__ void flush(double2& s, V4& a) {
   s.x += (double)a.h.x + (double)a.l.x;
   s.y += (double)a.h.y + (double)a.l.y;
   a = zero4();
-}
-
-__device__ __forceinline__ void upper_tile(int t, int ntile, int& ta, int& tc) {  // pairs ta <= tc, row by row
-  ta = 0;
-  while (t >= ntile - ta) {
-    t -= ntile - ta;
-    ++ta;
-  }
-  tc = ta + t;
-}
-
-template <bool RR, bool LL>
-__device__ __forceinline__ void proj_stage(const float4 (*sa)[kT], const float4 (*sr)[kT], const float4 (*sl)[kT],
-                                           int tx, int ty, V4 (&ar)[2][2], V4 (&al)[2][2]) {
-#pragma unroll 2
-  for (int k = 0; k < kK; ++k) {
-    V4 xa[2], xr[2], xl[2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      xa[i] = ld(sa[k][ty + 16 * i]);
-      if (RR) xr[i] = ld(sr[k][tx + 16 * i]);
-      if (LL) xl[i] = ld(sl[k][tx + 16 * i]);
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        if (RR) cmacc(ar[i][j], xa[i], xr[j]);
-        if (LL) cmacc(al[i][j], xa[i], xl[j]);
-      }
-  }
-}
-
-// part[s][which][a][c]: rows of chunk s; which = 0 (Gamma_R), 1 (Gamma_L).  A
-// stage in which one absorber's products all split to zero (rows far inside its
-// Gaussian's tail, below the range of a float) adds nothing and is passed over.
-__global__ void __launch_bounds__(kThr, 2)
-    proj_ds_kernel(const double2* __restrict__ U, int n, long long N, const double* __restrict__ gR,
-                   const double* __restrict__ gL, long long rch, int ntile, double2* __restrict__ part) {
-  __shared__ float4 sa[kK][kT], sr[kK][kT], sl[kK][kT];  // U[r][a], (Gamma U)[r][c]
-  int ta, tc;
-  upper_tile(blockIdx.x, ntile, ta, tc);
-  const int a0 = ta * kT, c0 = tc * kT;
-  const long long rb = (long long)blockIdx.y * rch, re = min(N, rb + rch);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  V4 ar[2][2], al[2][2];
-  double2 tr[2][2], tl[2][2];
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      ar[i][j] = al[i][j] = zero4();
-      tr[i][j] = tl[i][j] = make_double2(0.0, 0.0);
-    }
-  int stage = 0;
-  for (long long r0 = rb; r0 < re; r0 += kK) {
-    unsigned any_r = 0, any_l = 0;
-#pragma unroll
-    for (int q = 0; q < kK * kT / kThr; ++q) {
-      const int e = threadIdx.x + q * kThr, k = e / kT, col = e % kT;  // column fastest: coalesced rows of U
-      const long long r = r0 + k;
-      float4 va = make_float4(0.f, 0.f, 0.f, 0.f), vr = va, vl = va;
-      if (r < re) {
-        const double2* Ur = U + r * n;
-        if (a0 + col < n) va = split4(__ldg(Ur + a0 + col));
-        if (c0 + col < n) {
-          const double2 u = __ldg(Ur + c0 + col);
-          const double x = __ldg(gR + r), y = __ldg(gL + r);
-          vr = split4(make_double2(x * u.x, x * u.y));
-          vl = split4(make_double2(y * u.x, y * u.y));
-        }
-      }
-      sa[k][col] = va;
-      sr[k][col] = vr;
-      sl[k][col] = vl;
-      any_r |= (__float_as_uint(vr.x) | __float_as_uint(vr.y)) << 1;  // a nonzero head
-      any_l |= (__float_as_uint(vl.x) | __float_as_uint(vl.y)) << 1;
-    }
-    const bool has_r = __syncthreads_or(any_r != 0), has_l = __syncthreads_or(any_l != 0);
-    if (has_r && has_l) proj_stage<true, true>(sa, sr, sl, tx, ty, ar, al);
-    else if (has_r) proj_stage<true, false>(sa, sr, sl, tx, ty, ar, al);
-    else if (has_l) proj_stage<false, true>(sa, sr, sl, tx, ty, ar, al);
-    __syncthreads();
-    if (++stage == kFlush) {
-      stage = 0;
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          flush(tr[i][j], ar[i][j]);
-          flush(tl[i][j], al[i][j]);
-        }
-    }
-  }
-  double2* P = part + (size_t)blockIdx.y * 2 * n * n;
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int a = a0 + ty + 16 * i;
-    if (a >= n) continue;
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int c = c0 + tx + 16 * j;
-      if (c >= n) continue;
-      flush(tr[i][j], ar[i][j]);
-      flush(tl[i][j], al[i][j]);
-      P[(size_t)a * n + c] = tr[i][j];
-      P[(size_t)(n + a) * n + c] = tl[i][j];
-    }
-  }
-}
-
-// R[k][l] = M_R[l][k], L[k][l] = M_L[l][k], W = R o L from the chunks' upper tiles
-// (a lower tile is the conjugate of its mirror), and R, L split into floats
-__global__ void proj_ds_reduce_kernel(const double2* __restrict__ part, int chunks, int n, double2* __restrict__ R,
-                                      double2* __restrict__ L, double2* __restrict__ W) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)n * n) return;
-  const int k = (int)(t / n), l = (int)(t % n);
-  const bool up = l / kT <= k / kT;  // M[l][k] lies in an upper tile
-  const int i = up ? l : k, j = up ? k : l;
-  double2 r = make_double2(0.0, 0.0), q = r;
-  for (int s = 0; s < chunks; ++s) {
-    const double2* P = part + (size_t)s * 2 * n * n;
-    r = cadd(r, P[(size_t)i * n + j]);
-    q = cadd(q, P[(size_t)(n + i) * n + j]);
-  }
-  if (!up) {
-    r.y = -r.y;
-    q.y = -q.y;
-  }
-  R[t] = r;
-  L[t] = q;
-  W[t] = cmul(r, q);
 }
 
 __global__ void split_kernel(const double2* __restrict__ src, long long n, float4* __restrict__ dst) {
@@ -447,29 +311,6 @@ __global__ void sum_parts_kernel(const double2* __restrict__ part, int parts, lo
 }
 
 }  // namespace
-
-// Row chunks of the projections: about three waves of two blocks per SM over the
-// upper tiles, a chunk of at least 256 rows, at most 64 (the partial matrices)
-int proj_ds_chunks(int n, long long N) {
-  const long long nt = (n + kT - 1) / kT, pairs = nt * (nt + 1) / 2;
-  const long long k = std::min<long long>({(6 * 152 + pairs - 1) / pairs, (N + 255) / 256, 64});
-  return (int)std::max<long long>(k, 1);
-}
-
-void launch_proj_ds(const double2* U, int n, long long N, const double* gR, const double* gL, double2* part,
-                    int chunks, double2* R, double2* L, double2* W, cudaStream_t s, long long* launches) {
-  if (n <= 0 || N <= 0) return;
-  const int nt = (n + kT - 1) / kT;
-  long long rch = (N + chunks - 1) / chunks;
-  rch = (rch + kK - 1) / kK * kK;
-  const int nch = (int)((N + rch - 1) / rch);
-  proj_ds_kernel<<<dim3((unsigned)(nt * (nt + 1) / 2), (unsigned)nch), kThr, 0, s>>>(U, n, N, gR, gL, rch, nt, part);
-  SWI_CHECK_LAUNCH();
-  const long long nn = (long long)n * n;
-  proj_ds_reduce_kernel<<<(unsigned)((nn + 127) / 128), 128, 0, s>>>(part, nch, n, R, L, W);
-  SWI_CHECK_LAUNCH();
-  if (launches) *launches += 2;
-}
 
 // Energy groups of the adjoint: about two waves of two blocks per SM over the
 // tiles, at most 64 groups (the partial matrices)
