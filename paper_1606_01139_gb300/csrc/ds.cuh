@@ -66,14 +66,27 @@ __device__ __forceinline__ void split_flush(double x, float& hi, float& lo) {
   lo = small ? 0.f : (sgn ? -t : t);
 }
 
-// The same for any magnitude that a float can hold, still without FP64: below
-// 2^-74 the exponent is raised by 64 first and the parts are scaled back (their
-// tails then lie in or below the float denormals); below 2^-138 to (0, 0).
+// The same for every double, still without FP64, for operands that a caller
+// hands in.  Below 2^-74 the exponent is raised by 80 first and the parts are
+// scaled back (what then falls below the float denormals is lost); in the largest
+// binade of a float it is lowered by one; what lies beyond becomes an infinity,
+// and an infinity or a NaN stays one.
 __device__ __forceinline__ void split_wide(double x, float& hi, float& lo) {
   unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const bool tiny = ((unsigned int)(b >> 52) & 0x7ffu) < 949u;
-  if (tiny) b += 64ull << 52;
-  const float back = tiny ? 5.421010862427522e-20f : 1.f;  // 2^-64
+  const unsigned int top = (unsigned int)(b >> 32), e = (top >> 20) & 0x7ffu;
+  if (e - 949u <= 200u) {
+    split_flush(x, hi, lo);
+    return;
+  }
+  if (e > 1150u) {
+    const bool nan = e == 0x7ffu && (b << 12) != 0;
+    hi = __uint_as_float((top & 0x80000000u) | (nan ? 0x7fc00000u : 0x7f800000u));
+    lo = 0.f;
+    return;
+  }
+  if (e == 1150u) b -= 1ull << 52;
+  else b += 80ull << 52;
+  const float back = e == 1150u ? 2.f : 8.271806125530277e-25f;  // 2^-80
   split_flush(__longlong_as_double((long long)b), hi, lo);
   hi *= back;
   lo *= back;

@@ -79,7 +79,7 @@ struct swi_ctx {
   DevMem V, G, gL, gR;
   DevMem V32, G32;  // FP32 copies for the complex64 stencil
   DevMem VG32;      // (V, Gamma) pairs with even row length, for the TMA-staged stencil
-  DevMem VGds;      // (V, Gamma) split into floats, for the double-single stencil
+  DevMem VGds;      // 8 (V, Gamma) split into floats, for the double-single stencil
   DevMem pad_ds;    // its padded, split copy of the vectors
   bool has_V = false, has_G = false;
   double maxabsV = 0.0, maxG = 0.0;

@@ -16,7 +16,9 @@
 // against 12 per neighbour when every term is its own product.  The weights are
 // the integers 831600 c_m (the common denominator of the 12th-order formula)
 // over 2^21: exact floats without tails; one double-single product by the common
-// factor ends the sum.  Real and imaginary parts go through packed FP32x2
+// factor ends the sum.  The copy holds X / 8, so that six neighbours at the top of
+// a float's range still have a sum; the factors of the last products are 8 times
+// the operator's.  Real and imaginary parts go through packed FP32x2
 // instructions, and nothing touches the FP64 pipe (ds::join_bits).  Neighbours
 // come from L1, read ahead as far as 128 registers allow (limits of 80 or 64 for
 // more warps measured within 5%).  Forms that staged a plane per barrier in shared memory and kept the 13 z values
@@ -39,6 +41,7 @@ namespace {
 
 constexpr int kR = 6;
 constexpr int kRowsY = 8, kThreadsDs = 32 * kRowsY;
+constexpr float kIn = 0.125f, kOut = 8.f;  // scale of the padded copy, and of the factors of its products
 // 831600 c_1 .. 831600 c_6, c = 12/7, -15/56, 10/189, -1/112, 2/1925, -1/16632, over 2^21
 __host__ __device__ constexpr float weight(int m) {
   return (m == 1 ? 1425600.f : m == 2 ? -222750.f : m == 3 ? 44000.f : m == 4 ? -7425.f : m == 5 ? 864.f : -50.f) /
@@ -94,7 +97,7 @@ __device__ __forceinline__ int ghost(int j, int n, bool zero, float& sgn) {
   return s;
 }
 
-// P[z + 6][y + 6][(x + 6) nc + c] = X split, ghosts filled in; a block per rows of
+// P[z + 6][y + 6][(x + 6) nc + c] = X / 8 split, ghosts filled in; a block per rows of
 // (y, z), lanes along (x, c).  Only the cells a 37-point cross reads are needed:
 // a row with two or more of its coordinates outside is skipped.
 __global__ void __launch_bounds__(256) pad_ds_kernel(const double2* __restrict__ X, int ldx, int nc, int nx, int ny,
@@ -126,6 +129,7 @@ __global__ void __launch_bounds__(256) pad_ds_kernel(const double2* __restrict__
       const double2 v = __ldg(src + (long long)sx * ldx + c);
       ds::split_wide(v.x, o.x, o.z);
       ds::split_wide(v.y, o.y, o.w);
+      s *= kIn;
       o = make_float4(s * o.x, s * o.y, s * o.z, s * o.w);
     }
     dst[f] = o;
@@ -134,7 +138,7 @@ __global__ void __launch_bounds__(256) pad_ds_kernel(const double2* __restrict__
 
 __global__ void __launch_bounds__(kThreadsDs, 2)
     stencil_ds_kernel(const float4* __restrict__ P, int nc, int nx, int ny, int nz, const float4* __restrict__ VG,
-                      const double* __restrict__ sigma, double cm0, float2 fac,  // c_m = (fac.x + fac.y) weight(m)
+                      const double* __restrict__ sigma, double cm0, float2 fac,  // 8 c_m = (fac.x + fac.y) weight(m)
                       double2* __restrict__ Y, int ldy, int out_ds, int zchunk) {
   const int xb = (nx * nc + 31) / 32;  // blocks along (x, c)
   const int f = (blockIdx.x % xb) * 32 + (threadIdx.x & 31), y = (blockIdx.x / xb) * kRowsY + (threadIdx.x >> 5);
@@ -144,8 +148,10 @@ __global__ void __launch_bounds__(kThreadsDs, 2)
   const int rowp = px * nc;                     // elements between y neighbours
   const long long planep = (long long)rowp * py;  // and between z neighbours
   const int z0 = blockIdx.y * zchunk, z1 = min(nz, z0 + zchunk);
-  ds::df dcen;  // 3 c_0 - sigma
+  ds::df dcen;  // 8 (3 c_0 - sigma)
   ds::split_wide(3.0 * cm0 - sigma[c], dcen.h, dcen.l);
+  dcen.h *= kOut;
+  dcen.l *= kOut;
   const float4* p = P + (long long)(z0 + kR) * planep + (long long)(y + kR) * rowp + (x + kR) * nc + c;
   for (int z = z0; z < z1; ++z, p += planep) {
     const long long r = ((long long)z * ny + y) * nx + x;
@@ -183,7 +189,7 @@ __global__ void pack_vg_ds_kernel(const double* __restrict__ V, const double* __
     float4 o;
     ds::split_bits(V[e], o.x, o.y);
     ds::split_bits(G[e], o.z, o.w);
-    out[e] = o;
+    out[e] = make_float4(kOut * o.x, kOut * o.y, kOut * o.z, kOut * o.w);
   }
 }
 
@@ -214,7 +220,7 @@ void launch_stencil_ds(const StencilParams& P, const double2* X, int ldx, double
   if (P.VGds == nullptr || work == nullptr)
     throw Error{SWI_ESTATE, "double-single stencil: the split (V, Gamma) array or the work space is missing"};
   const double fd = P.cm[1] / (double)weight(1);
-  const float2 fac = make_float2((float)fd, (float)(fd - (double)(float)fd));
+  const float2 fac = make_float2(kOut * (float)fd, kOut * (float)(fd - (double)(float)fd));
   const int px = P.nx + 2 * kR;
   const long long rows = (long long)(P.ny + 2 * kR) * (P.nz + 2 * kR);
   const int step = pass_columns(P, ncols);

@@ -88,7 +88,7 @@ struct StencilParams {
   double cm[7];       // -c_m / (2 h^2), m = 0..6 (centre weight counts once per axis)
   const double* V;    // N
   const double* G;    // Gamma_L + Gamma_R, N
-  const float4* VGds; // (V head, V tail, Gamma head, Gamma tail), N (the double-single kernel)
+  const float4* VGds; // 8 x (V head, V tail, Gamma head, Gamma tail), N (the double-single kernel)
 };
 void launch_pack_vg_ds(const double* V, const double* G, long long n, float4* out, cudaStream_t s);
 
