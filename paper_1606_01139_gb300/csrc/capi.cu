@@ -1629,7 +1629,7 @@ swi_status swi_grad(swi_ctx* c, int nE, const double* E, const double* dLdT, dou
       if (c->arith != SWI_ARITH_F64) {
         const size_t nn = (size_t)n * n;
         const int groups = swi::gradM_ds_groups(n, nE);
-        c->gsplit.ensure(sizeof(float4) * (2 * nn + (size_t)nE * n + 1));
+        c->gsplit.ensure(sizeof(float4) * swi::gradM_ds_split(n, nE));
         gram_work_ensure(c, nn * (size_t)groups);
         swi::launch_gradM_ds(c->Rm.as<double2>(), c->Lm.as<double2>(), c->eps.as<double2>(), n, c->Ebuf.as<double>(),
                              c->wbuf.as<double>(), nE, groups, c->gsplit.as<float4>(), c->gram_work.as<double2>(),

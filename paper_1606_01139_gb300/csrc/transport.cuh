@@ -25,9 +25,11 @@ void launch_grad_f32(const float2* R32, const float2* L32, const double2* eps, i
                      const double* w, int nE, float2* gt, float2* M, float2* S, const double2* U, int ldu, long long N,
                      double* out, cudaStream_t s, long long* launches);
 // Double-single contractions of the adjoint (transport_ds.cu).
-// M = sum_e w_e D_e R conj(D_e) L^T D_e; split: 2 n^2 + nE n entries of scratch,
-// part: gradM_ds_groups(n, nE) matrices of n x n
+// M = sum_e w_e D_e R conj(D_e) L^T D_e; split: gradM_ds_split(n, nE) entries of
+// scratch (R, L, the energy table, the rows' scales), part: gradM_ds_groups(n, nE)
+// matrices of n x n
 int gradM_ds_groups(int n, int nE);
+inline size_t gradM_ds_split(int n, int nE) { return 2 * (size_t)n * n + (size_t)nE * n + (size_t)n; }
 void launch_gradM_ds(const double2* R, const double2* L, const double2* eps, int n, const double* E, const double* w,
                      int nE, int groups, float4* split, double2* part, double2* M, cudaStream_t s,
                      long long* launches);

@@ -79,9 +79,36 @@ __device__ __forceinline__ void flush(double2& s, V4& a) {
   a = zero4();
 }
 
-__global__ void split_kernel(const double2* __restrict__ src, long long n, float4* __restrict__ dst) {
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
-    dst[e] = split4(src[e]);
+// A power of two that brings a largest magnitude (its bits) to [1, 2) (1 where
+// there is none, or no finite one), and its inverse: weakly coupled wires have
+// projections and an M far below 1, whose products would leave the range of a float.
+__device__ __forceinline__ double unit_scale(unsigned long long mx, bool inverse) {
+  const unsigned ef = (unsigned)(mx >> 52);
+  if (ef == 0 || ef >= 0x7ff) return 1.0;
+  const unsigned f = max(2046u - ef, 1u);
+  return __longlong_as_double((long long)(inverse ? 2046u - f : f) << 52);
+}
+__device__ __forceinline__ unsigned long long max_bits(unsigned long long v, double2 m) {
+  return max(v, max((unsigned long long)__double_as_longlong(fabs(m.x)), (unsigned long long)__double_as_longlong(fabs(m.y))));
+}
+
+// R and L (blockIdx.y) scaled by rows and split, a warp per row; inv[row]: the
+// inverse of the row's scale (R first, then L).  Both are linear in the absorbers:
+// a row of 1e-20 against one of L of 1e-20 has products that no float holds.
+__global__ void __launch_bounds__(kThr) split_rows_kernel(const double2* __restrict__ R, const double2* __restrict__ L,
+                                                         int n, float4* __restrict__ Rs, float4* __restrict__ Ls,
+                                                         double* __restrict__ inv) {
+  const int row = blockIdx.x * (kThr / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (row >= n) return;
+  const double2* src = (blockIdx.y ? L : R) + (size_t)row * n;
+  float4* dst = (blockIdx.y ? Ls : Rs) + (size_t)row * n;
+  unsigned long long v = 0;
+  for (int l = lane; l < n; l += 32) v = max_bits(v, src[l]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  const double f = unit_scale(v, false);
+  for (int l = lane; l < n; l += 32) dst[l] = split4(cscale(src[l], f));
+  if (lane == 0) inv[blockIdx.y * n + row] = unit_scale(v, true);
 }
 
 // gt[e][l] = 1/(E_e - eps_l), formed in FP64 and split
@@ -93,10 +120,12 @@ __global__ void gtab_ds_kernel(const double2* __restrict__ eps, int n, const dou
   gt[t] = split4(cdiv(make_double2(1.0, 0.0), csub(make_double2(E[e], 0.0), eps[l])));
 }
 
-// part[s][a][c] = the energies of group s (blockIdx.z) of M
+// part[s][a][c] = the energies of group s (blockIdx.z) of M, from the rows of R and
+// L as they are scaled
 __global__ void __launch_bounds__(kThr, 2)
     gradM_ds_kernel(const float4* __restrict__ R, const float4* __restrict__ L, const float4* __restrict__ gt,
-                    const double* __restrict__ wts, int n, int nE, int per, double2* __restrict__ part) {
+                    const double* __restrict__ inv, const double* __restrict__ wts, int n, int nE, int per,
+                    double2* __restrict__ part) {
   __shared__ float4 sr[kK][kT + 1], sl[kK][kT + 1];  // R[a][l], conj(g_l) L[c][l]
   const int a0 = blockIdx.y * kT, c0 = blockIdx.x * kT;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -184,7 +213,7 @@ __global__ void __launch_bounds__(kThr, 2)
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       const int c = c0 + tx + 16 * j;
-      if (c < n) P[(size_t)a * n + c] = tot[i][j];
+      if (c < n) P[(size_t)a * n + c] = cscale(cscale(tot[i][j], inv[a]), inv[n + c]);
     }
   }
 }
@@ -193,22 +222,11 @@ __global__ void __launch_bounds__(kThr, 2)
 __global__ void absmax_kernel(const double2* __restrict__ M, long long nn, unsigned long long* __restrict__ mx) {
   unsigned long long v = 0;
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < nn; t += (long long)gridDim.x * blockDim.x) {
-    const double2 m = M[t];
-    v = max(v, max((unsigned long long)__double_as_longlong(fabs(m.x)), (unsigned long long)__double_as_longlong(fabs(m.y))));
+    v = max_bits(v, M[t]);
   }
   for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
   if ((threadIdx.x & 31) == 0 && v) atomicMax(mx, v);
 }
-// a power of two that brings M's largest entry to about 1 (1 where there is none,
-// or no finite one), and its inverse: weakly coupled wires have an M far below 1,
-// whose products with small entries of U would leave the range of a float
-__device__ __forceinline__ double m_scale(unsigned long long mx, bool inverse) {
-  const unsigned ef = (unsigned)(mx >> 52);
-  if (ef == 0 || ef >= 0x7ff) return 1.0;
-  const unsigned f = max(2046u - ef, 1u);
-  return __longlong_as_double((long long)(inverse ? 2046u - f : f) << 52);
-}
-
 // S[a][c] scaled and split, a <= c (zero below the diagonal)
 __global__ void symsplit_kernel(const double2* __restrict__ M, int n, const unsigned long long* __restrict__ mx,
                                 float4* __restrict__ S) {
@@ -218,7 +236,7 @@ __global__ void symsplit_kernel(const double2* __restrict__ M, int n, const unsi
   double2 v = make_double2(0.0, 0.0);
   if (a <= c) v = M[t];
   if (a < c) v = cadd(v, M[(size_t)c * n + a]);
-  S[t] = split4(cscale(v, m_scale(*mx, false)));
+  S[t] = split4(cscale(v, unit_scale(*mx, false)));
 }
 
 // out[r] for the 32 rows r0 .. r0 + 31 of a block: per 32-column tile the sums
@@ -297,7 +315,7 @@ __global__ void __launch_bounds__(kThr, 2)
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const long long r = r0 + ty + 16 * i;
-      if (r < N) out[r] = 2.0 * m_scale(*mx, true) * row[i];
+      if (r < N) out[r] = 2.0 * unit_scale(*mx, true) * row[i];
     }
   }
 }
@@ -326,23 +344,21 @@ void launch_gradM_ds(const double2* R, const double2* L, const double2* eps, int
   if (n <= 0) return;
   const long long nn = (long long)n * n, ne = (long long)nE * n;
   float4 *Rs = split, *Ls = split + nn, *gt = split + 2 * nn;
-  const unsigned gs = (unsigned)std::min<long long>((nn + 255) / 256, 4096);
-  split_kernel<<<gs, 256, 0, s>>>(R, nn, Rs);
-  SWI_CHECK_LAUNCH();
-  split_kernel<<<gs, 256, 0, s>>>(L, nn, Ls);
+  double* inv = reinterpret_cast<double*>(gt + ne);
+  split_rows_kernel<<<dim3((unsigned)((n + kThr / 32 - 1) / (kThr / 32)), 2), kThr, 0, s>>>(R, L, n, Rs, Ls, inv);
   SWI_CHECK_LAUNCH();
   gtab_ds_kernel<<<(unsigned)((ne + 255) / 256), 256, 0, s>>>(eps, n, E, nE, gt);
   SWI_CHECK_LAUNCH();
   const unsigned nt = (unsigned)((n + kT - 1) / kT);
   const int per = (nE + groups - 1) / groups, ng = (nE + per - 1) / per;
   double2* dst = ng > 1 ? part : M;
-  gradM_ds_kernel<<<dim3(nt, nt, (unsigned)ng), kThr, 0, s>>>(Rs, Ls, gt, w, n, nE, per, dst);
+  gradM_ds_kernel<<<dim3(nt, nt, (unsigned)ng), kThr, 0, s>>>(Rs, Ls, gt, inv, w, n, nE, per, dst);
   SWI_CHECK_LAUNCH();
   if (ng > 1) {
     sum_parts_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(part, ng, nn, M);
     SWI_CHECK_LAUNCH();
   }
-  if (launches) *launches += ng > 1 ? 5 : 4;
+  if (launches) *launches += ng > 1 ? 4 : 3;
 }
 
 void launch_rowquad_ds(const double2* U, const double2* M, int n, long long N, float4* split, double* out,
