@@ -241,7 +241,9 @@ __global__ void symsplit_kernel(const double2* __restrict__ M, int n, const unsi
 
 // out[r] for the 32 rows r0 .. r0 + 31 of a block: per 32-column tile the sums
 // over a <= c, contracted with the same rows of U at once (nothing of size N x n
-// is stored)
+// is stored).  LONG, past kFlush stages: a tile is contracted after every kFlush
+// of them (the loop alone costs the short form 2.5%)
+template <bool LONG>
 __global__ void __launch_bounds__(kThr, 2)
     rowquad_ds_kernel(const double2* __restrict__ U, const float4* __restrict__ S, int n, long long N,
                       const unsigned long long* __restrict__ mx, double* __restrict__ out) {
@@ -250,14 +252,15 @@ __global__ void __launch_bounds__(kThr, 2)
   const long long r0 = (long long)blockIdx.x * kT;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   double row[2] = {0.0, 0.0};
-  for (int c0 = 0; c0 < n; c0 += kT) {
+  for (int c0 = 0; c0 < n; c0 += kT)
+  for (int as = 0, end = min(n, c0 + kT); as < (LONG ? end : 1); as += kFlush * kK) {
     V4 acc[2][2];
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int j = 0; j < 2; ++j) acc[i][j] = zero4();
-    const int a1 = min(n, c0 + kT);
-    for (int a0 = 0; a0 < a1; a0 += kK) {
+    const int a1 = LONG ? min(end, as + kFlush * kK) : end;
+    for (int a0 = as; a0 < a1; a0 += kK) {
 #pragma unroll
       for (int q = 0; q < kK * kT / kThr; ++q) {
         const int f = threadIdx.x + q * kThr;
@@ -288,7 +291,7 @@ __global__ void __launch_bounds__(kThr, 2)
       }
       __syncthreads();
     }
-    // Re(acc U[r][c]), one FP64 addition per row and tile
+    // Re(acc U[r][c]), one FP64 addition per row, tile and 1,024 terms
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const long long r = r0 + ty + 16 * i;
@@ -371,7 +374,9 @@ void launch_rowquad_ds(const double2* U, const double2* M, int n, long long N, f
   SWI_CHECK_LAUNCH();
   symsplit_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(M, n, mx, split);
   SWI_CHECK_LAUNCH();
-  rowquad_ds_kernel<<<(unsigned)((N + kT - 1) / kT), kThr, 0, s>>>(U, split, n, N, mx, out);
+  const unsigned grid = (unsigned)((N + kT - 1) / kT);
+  if (n > kFlush * kK) rowquad_ds_kernel<true><<<grid, kThr, 0, s>>>(U, split, n, N, mx, out);
+  else rowquad_ds_kernel<false><<<grid, kThr, 0, s>>>(U, split, n, N, mx, out);
   SWI_CHECK_LAUNCH();
   if (launches) *launches += 3;
 }

@@ -1,5 +1,5 @@
 """Adjoint of T(E) in double-single where its operands leave the range of a float: absorbers so weak that the products
-of the projections would vanish, on one side or both.
+of the projections would vanish, on one side or both; and sums past the 1,024 terms that stay in double-single.
 
 Bounds as in test_zzz_transport_ds.py: a double-single product is exact to 2^-47 of its magnitude, a chain of k
 additions to k 2^-48 of the sum of the magnitudes (k at most 1,100 before the FP64 sums)."""
@@ -42,4 +42,11 @@ def _adjoint(n, nE, sL, sR, shape):
 def test_weak_absorbers(sL, sR):
     dV, want, tol = _adjoint(37, 5, sL, sR, (7, 6, 63))
     assert np.abs(want).max() > 0
+    assert np.all(np.abs(dV - want) <= tol)
+
+
+# a tile of 32 pairs, then one pair, past the limit; 1,176 rows
+@pytest.mark.parametrize("n,nE", [(1056, 1), (1025, 2)])
+def test_long_sums(n, nE):
+    dV, want, tol = _adjoint(n, nE, 1.0, 1.0, (6, 7, 28))
     assert np.all(np.abs(dV - want) <= tol)
