@@ -127,9 +127,12 @@ typedef struct {
   int restarts;
   int basis;            /* m_j used */
   double max_res;       /* largest relative residual of the delivered pairs */
-  int schur_retries;    /* restarts whose double-single Schur step gave up and
-                           were recomputed in native FP64 */
-  int reserved;
+  int schur_retries;    /* restarts whose double-single Schur step of full
+                           order gave up and were recomputed in native FP64 */
+  int schur_fallbacks;  /* restarts whose first form of the Schur step (FP32
+                           Schur form, kept subspace corrected to
+                           double-single) gave up and were recomputed by the
+                           double-single step of full order */
 } swi_window_info;
 
 typedef struct {
@@ -530,6 +533,19 @@ swi_status swi_transmission_noalloc(swi_ctx* ctx, int nE, const double* E, doubl
  * (m outside 2..1024, b, keep outside 1..m-b, NULL), SWI_ECUDA. */
 swi_status swi_check_schur(swi_ctx* ctx, int m, int b, int keep, const double* H, const double* B, int arith,
                            double* T_out, double* Z_out, int* info_out);
+
+/* The same check of the form that a restart tries first: an FP32 Schur form,
+ * the kept subspace corrected to double-single accuracy (orders 48..512,
+ * SWI_ARITH_DS).  It determines the k kept columns alone: T_out holds the k x k
+ * triangular block in its leading corner, Z_out the k Schur vectors in its first
+ * columns (H Z = Z T), zeros elsewhere.  n_want: wanted values among the kept
+ * (1..keep); sig_im: the kept values are those of smallest |theta - i sig_im|.
+ * b up to 32.  info_out[4]: kept columns (keep or a few more at a tie),
+ * wanted pairs whose residual estimate is 0, status (0 done, 1 gave up: the
+ * solver then runs the full-order step), work.  Errors: SWI_EINVAL (sizes that
+ * this form does not take, NULL), SWI_ECUDA. */
+swi_status swi_check_restart(swi_ctx* ctx, int m, int b, int keep, int n_want, double sig_im, const double* H,
+                             const double* B, double* T_out, double* Z_out, int* info_out);
 
 /* Message of the last failing call on ctx (thread-local for ctx == NULL). */
 const char* swi_last_error(const swi_ctx* ctx);

@@ -31,7 +31,7 @@ EXPORTS = ("swi_create", "swi_set_potential", "swi_set_absorber", "swi_set_windo
            "swi_apply", "swi_apply_ds", "swi_apply_c64", "swi_solve", "swi_solve_batch", "swi_solve_more", "swi_fill_holes",
            "swi_get_windows", "swi_refine", "swi_get_window_info", "swi_get_eigenpairs", "swi_copy_eigenpairs",
            "swi_set_eigenpairs", "swi_residuals", "swi_transmission", "swi_set_contraction", "swi_grad", "swi_profile",
-           "swi_profile_read", "swi_transmission_noalloc", "swi_check_schur", "swi_last_error", "swi_launch_count",
+           "swi_profile_read", "swi_transmission_noalloc", "swi_check_schur", "swi_check_restart", "swi_last_error", "swi_launch_count",
            "swi_destroy")
 
 KERNEL_CLASSES = ("stencil", "gram", "update", "cholqr", "schur", "rotate", "merge", "proj", "trans", "grad")
@@ -79,7 +79,7 @@ class PlanInfo(C.Structure):
 class WindowInfo(C.Structure):
     _fields_ = [("sigma", C.c_double), ("n_req", C.c_int), ("n_conv", C.c_int), ("matvecs", C.c_longlong),
                 ("restarts", C.c_int), ("basis", C.c_int), ("max_res", C.c_double), ("schur_retries", C.c_int),
-                ("reserved", C.c_int)]
+                ("schur_fallbacks", C.c_int)]
 
 
 class SolveInfo(C.Structure):
@@ -132,6 +132,7 @@ def load(path: str = LIB_PATH):
         "swi_profile": (I, [VP, I]),
         "swi_transmission_noalloc": (I, [VP, I, VP, VP]),
         "swi_check_schur": (I, [VP, I, I, I, VP, VP, I, VP, VP, VP]),
+        "swi_check_restart": (I, [VP, I, I, I, I, D, VP, VP, VP, VP, VP]),
         "swi_profile_read": (I, [VP, P(KernelStats)]),
         "swi_last_error": (C.c_char_p, [VP]),
         "swi_launch_count": (C.c_longlong, [VP]),
@@ -435,6 +436,22 @@ class Context:
         self._check(self._lib.swi_check_schur(self._h, m, b, keep, _ptr(H), None if Bc is None else _ptr(Bc), int(arith),
                                               _ptr(T), _ptr(Z), _ptr(info)))
         return T, Z, info
+
+    def check_restart(self, H, B=None, keep=None, n_want=1, sig_im=0.0):
+        """The form of the Schur step that a restart tries first, on a host matrix H (m x m): (T [k, k], Z [m, k], info)
+        with H Z = Z T for the k = info[0] kept values; info = (kept, -, status, work), status 1: it gave up."""
+        H = _c_arr(np.asarray(H), np.complex128)
+        m = H.shape[0]
+        b = 1 if B is None else np.atleast_2d(B).shape[0]
+        Bc = None if B is None else _c_arr(np.atleast_2d(B), np.complex128)
+        keep = m // 2 if keep is None else int(keep)
+        T = np.empty((m, m), np.complex128)
+        Z = np.empty((m, m), np.complex128)
+        info = np.zeros(4, np.int32)
+        self._check(self._lib.swi_check_restart(self._h, m, b, keep, int(n_want), float(sig_im), _ptr(H),
+                                                None if Bc is None else _ptr(Bc), _ptr(T), _ptr(Z), _ptr(info)))
+        k = int(info[0])
+        return T[:k, :k], Z[:, :k], info
 
     def grad(self, E, dLdT, dLdV_out=None):
         """(dL/dV[N], dL/dE[nE]) for the weights dL/dT (dL/dE_e = dLdT_e dT_e/dE_e).

@@ -513,6 +513,7 @@ swi_status do_solve(swi_ctx* c, const swi_solve_opts* o, swi_solve_info* info) {
     const int* oi = side.oi + 4 * j;
     const int k = oi[0], nconv = oi[1], st = oi[2];
     if (st != 0 && c->arith != SWI_ARITH_F64 && !w.retried) {
+      w.schur_fallbacks++;
       launch_schur(j, true);
       return;
     }
@@ -698,6 +699,7 @@ swi_status do_solve(swi_ctx* c, const swi_solve_opts* o, swi_solve_info* info) {
     double mr = 0.0;
     for (double r : rw) mr = std::max(mr, r / anorm);
     wi.max_res = mr;
+    wi.schur_fallbacks = w.schur_fallbacks;
     any_fail |= w.failed;
     any_noconv |= (w.nconv < w.nreq);
   }
@@ -1781,6 +1783,45 @@ swi_status swi_check_schur(swi_ctx* c, int m, int b, int keep, const double* H, 
     SWI_CUDA_TRY(cudaMemcpyAsync(Z_out, dZ.p, sizeof(double2) * mm, cudaMemcpyDeviceToHost, c->stream));
     SWI_CUDA_TRY(cudaMemcpyAsync(info_out, dinfo.p, sizeof(int) * 4, cudaMemcpyDeviceToHost, c->stream));
     sync(c->stream);
+    return SWI_OK;
+  });
+}
+
+swi_status swi_check_restart(swi_ctx* c, int m, int b, int keep, int n_want, double sig_im, const double* H,
+                             const double* B, double* T_out, double* Z_out, int* info_out) {
+  return guarded(c, [&]() -> swi_status {
+    if (m < 2 || b < 1 || b > 32 || keep < 1 || keep > m - b || n_want < 1 || n_want > keep || !H || !T_out ||
+        !Z_out || !info_out || !swi::mp_schur_takes(m, keep, m - b) || !std::isfinite(sig_im))
+      return fail(c, SWI_EINVAL, "check_restart: bad arguments");
+    const size_t mm = (size_t)m * m;
+    const int kcap = std::min(keep + 8, m - b);
+    DevMem dH, dZ, dB, dBz, dth, dres, dS, dinfo, dwork;
+    dH.ensure(sizeof(double2) * mm);
+    dZ.ensure(sizeof(double2) * mm);
+    dS.ensure(sizeof(double2) * mm);
+    dB.ensure(sizeof(double2) * b * m);
+    dBz.ensure(sizeof(double2) * b * m);
+    dth.ensure(sizeof(double2) * m);
+    dres.ensure(sizeof(double) * m);
+    dinfo.ensure(sizeof(int) * 4);
+    dwork.ensure(swi::mp_schur_bytes(m, kcap, m, b));
+    SWI_CUDA_TRY(cudaMemcpyAsync(dH.p, H, sizeof(double2) * mm, cudaMemcpyHostToDevice, c->stream));
+    if (B) SWI_CUDA_TRY(cudaMemcpyAsync(dB.p, B, sizeof(double2) * b * m, cudaMemcpyHostToDevice, c->stream));
+    else SWI_CUDA_TRY(cudaMemsetAsync(dB.p, 0, sizeof(double2) * b * m, c->stream));
+    SWI_CUDA_TRY(cudaMemsetAsync(dZ.p, 0, sizeof(double2) * mm, c->stream));
+    const swi::SchurJob job{dH.as<double2>(), dZ.as<double2>(), dB.as<double2>(), dBz.as<double2>(),
+                            dth.as<double2>(), dres.as<double>(), dS.as<double2>(), dinfo.as<int>(),
+                            m, m, b, keep, n_want, m - b, 0.0, nullptr, nullptr, sig_im};
+    swi::launch_schur_mp(job, dwork.p, kcap, c->stream, &c->launches);
+    SWI_CUDA_TRY(cudaMemcpyAsync(T_out, dH.p, sizeof(double2) * mm, cudaMemcpyDeviceToHost, c->stream));
+    SWI_CUDA_TRY(cudaMemcpyAsync(Z_out, dZ.p, sizeof(double2) * mm, cudaMemcpyDeviceToHost, c->stream));
+    SWI_CUDA_TRY(cudaMemcpyAsync(info_out, dinfo.p, sizeof(int) * 4, cudaMemcpyDeviceToHost, c->stream));
+    sync(c->stream);
+    const int k = info_out[2] == 0 ? info_out[0] : 0;  // the rest of H is as it came in
+    double2* T = reinterpret_cast<double2*>(T_out);
+    for (int i = 0; i < m; ++i)
+      for (int j = 0; j < m; ++j)
+        if (i >= k || j >= k) T[(size_t)i * m + j] = make_double2(0.0, 0.0);
     return SWI_OK;
   });
 }

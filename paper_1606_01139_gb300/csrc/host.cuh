@@ -61,7 +61,7 @@ struct Window {
   int cur = 0, p = 0;
   bool done = false, failed = false, retried = false;
   long long matvecs = 0;
-  int restarts = 0;
+  int restarts = 0, schur_fallbacks = 0;
   int nconv = 0;
   double max_res = 0.0;
 };

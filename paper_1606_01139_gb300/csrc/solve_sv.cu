@@ -60,7 +60,7 @@ struct SvWin {
   DevMem Hsave;          // the projected matrix of the Schur step in flight (for a retry)
   DevMem mpw;            // work of the restart's form of the step (schur_mp.cu)
   int form = 0;          // kernel of the Schur step in flight: kFormMp, kFormDs or kFormF64
-  int schur_retries = 0;
+  int schur_retries = 0, schur_fallbacks = 0;
   bool done = false, failed = false;
   long long matvecs = 0;
   int restarts = 0, nconv = 0;
@@ -381,6 +381,7 @@ swi_status solve_sv(swi_ctx* c, const swi_solve_opts& opt, swi_solve_info* info)
     const int n = w.p;  // order of the projected matrix
     if (st != 0 && w.form < kFormF64) {  // it gave up: the next form on the same matrix
       if (w.form == kFormDs) w.schur_retries++;
+      else w.schur_fallbacks++;
       launch_schur(w, w.form + 1);
       return;
     }
@@ -561,6 +562,7 @@ swi_status solve_sv(swi_ctx* c, const swi_solve_opts& opt, swi_solve_info* info)
     for (double r : rw) mr = std::max(mr, r / anorm);
     wi.max_res = mr;
     wi.schur_retries = w.schur_retries;
+    wi.schur_fallbacks = w.schur_fallbacks;
     double2 flag;
     SWI_CUDA_TRY(cudaMemcpy(&flag, w.rinv.template as<double2>() + 8, sizeof(double2), cudaMemcpyDeviceToHost));
     if (flag.x != 0.0) any_breakdown = true;
