@@ -31,9 +31,10 @@
 // 163-184 (35-110 kept); |H Z - Z T| / max|H| 0.6-2e-14, |Z^H Z - I| 2e-14 to
 // 2e-13 on restart matrices of orders 150-208.
 //
-// A failure (iteration or list limit, corrections that do not converge) is
-// reported as status 1 in ordinfo[2]; the caller then runs the double-single
-// kernel of order m on the saved matrix.
+// A failure (iteration or list limit, corrections that do not converge, a last
+// restart whose kept set hangs on FP32 rounding) is reported as status 1 in
+// ordinfo[2]; the caller then runs the double-single kernel of order m on the
+// saved matrix.
 #include <mutex>
 #include <set>
 #include <type_traits>
@@ -1150,6 +1151,7 @@ __global__ void __launch_bounds__(512, 1) mp_order_kernel(const __grid_constant_
   }
   if (in_smem)
     for (int e = tid; e < offu(m); e += 512) J.T[e] = T[e];
+  if (tid < m) J.rad[tid] = sorted[tid];
   for (int i = warp; i < m; i += 16)
     for (int j = i + lane; j < m; j += 32) J.Tr[row_at(m, i) + j - i] = T[offu(j) + i];
   if (tid == 0) {
@@ -1304,11 +1306,23 @@ __global__ void mp_couple_kernel(const __grid_constant__ MpJob J, const double2*
   }
 }
 
-// the step's outcome: kept count, wanted pairs at the tolerance, status, work
+// The step's outcome: kept count, wanted pairs at the tolerance, status, work.
+// The kept set was chosen by FP32 values.  When all wanted pairs are at the
+// tolerance (the window would end), the nearest value left out must lie beyond
+// the last wanted one by more than those values are off: 16 times the largest
+// change of a kept value's distance between the two forms (values of the same
+// matrix, of conditions that differ).  If not, the step gives up, and the
+// full-order step decides.
 __global__ void __launch_bounds__(512) mp_outcome_kernel(const __grid_constant__ MpJob J) {
   __shared__ int s_n;
+  __shared__ unsigned s_off;
+  __shared__ double s_last;
   const int k0 = J.ctl[CTL_K0], st = J.ctl[CTL_STATUS];
-  if (threadIdx.x == 0) s_n = 0;
+  if (threadIdx.x == 0) {
+    s_n = 0;
+    s_off = 0u;
+    s_last = 0.0;
+  }
   __syncthreads();
   if (st == 0)
     for (int i = threadIdx.x; i < k0; i += blockDim.x) {
@@ -1321,12 +1335,16 @@ __global__ void __launch_bounds__(512) mp_outcome_kernel(const __grid_constant__
         if (aq < ai || (aq == ai && q < i)) ++rank;
       }
       if (rank < J.nwant && J.resid[i] <= J.tol_abs) atomicAdd(&s_n, 1);
+      if (rank == J.nwant - 1) s_last = ai;
+      atomicMax(&s_off, __float_as_uint((float)fabs(ai - (double)J.rad[rank])));
     }
   __syncthreads();
   if (threadIdx.x == 0) {
+    const bool unsure = st == 0 && s_n >= J.nwant && k0 < J.m &&
+                        !((double)J.rad[k0] - 16.0 * (double)__uint_as_float(s_off) > s_last);
     J.ordinfo[0] = k0;
     J.ordinfo[1] = s_n;
-    J.ordinfo[2] = st != 0 ? 1 : 0;
+    J.ordinfo[2] = st != 0 || unsure ? 1 : 0;
     J.ordinfo[3] = (int)(((long long)J.ctl[CTL_STEPSK] * 4 * 2 * k0) >> 10);  // Givens pair updates / 1024
   }
 }
@@ -1374,6 +1392,7 @@ size_t mp_schur_layout(MpJob* J, void* base, int m, int kcap, int ld, int b) {
   t.Hp = static_cast<float2*>(take(8 * (size_t)offh(m)));
   t.Vr = static_cast<float2*>(take(8 * mm));
   t.tau = static_cast<float*>(take(4 * (size_t)m));
+  t.rad = static_cast<float*>(take(4 * (size_t)m));
   t.len = static_cast<int*>(take(4 * (size_t)m));
   t.Q = static_cast<float2*>(take(8 * mm));
   t.P = static_cast<float2*>(take(8 * mm));

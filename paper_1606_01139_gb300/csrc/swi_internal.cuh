@@ -237,7 +237,7 @@ struct MpJob {
   int* ordinfo;
   int* ctl;                                                // control block (enum CTL_*)
   float2 *H32, *Hp, *Vr, *Q, *P, *T, *Tr, *R32, *X, *S32;       // FP32 work
-  float* tau;
+  float *tau, *rad;                                        // rad: the FP32 form's |theta - i sig_im|, ascending
   int* len;                                                // rows of each reflector
   float4 *rot, *rot2, *rotk;                               // rotation lists
   double2 *V[2], *W, *G, *BV;
