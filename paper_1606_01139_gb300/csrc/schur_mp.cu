@@ -132,8 +132,8 @@ struct Arith<dc> {
   using R = df;
   __device__ static dc from(double2 v) {
     dc r;
-    ds::split_flush(v.x, r.re.h, r.re.l);
-    ds::split_flush(v.y, r.im.h, r.im.l);
+    ds::split_wide(v.x, r.re.h, r.re.l);
+    ds::split_wide(v.y, r.im.h, r.im.l);
     return r;
   }
   __device__ static dc zero() { return ds::czero(); }
@@ -260,6 +260,7 @@ __device__ __forceinline__ Rot make_rot(float2 x, float2 y, float2& r) {
   }
   return g;
 }
+__device__ __forceinline__ float2 scale_f(float2 a, float t) { return fc(a.x * t, a.y * t); }
 __device__ __forceinline__ dc scale_f(dc a, float t) {
   return dc{df{a.re.h * t, a.re.l * t}, df{a.im.h * t, a.im.l * t}};
 }
@@ -374,7 +375,10 @@ __device__ __forceinline__ int order_of(int order, const int* ctl) { return orde
 // memory.  Per column: the reflector, its left product (thread groups over row
 // classes, summed in shared memory), then one pass over the rows (a warp per
 // row, the row in registers) that applies the left update, forms the right
-// product and applies it.  NT x 32 >= the order.
+// product and applies it.  NT x 32 >= the order.  The matrix is scaled to order
+// one (pow2_scales of its largest entry; the reflectors and the chase's rotations
+// do not see the scale): only squares of entries far below rounding leave the
+// float range then, whatever the size of H.
 template <class C, int NT, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1) mp_hess_kernel(const __grid_constant__ Red<C> D, int* ctl, int in_smem) {
   using R = typename Arith<C>::R;
@@ -394,6 +398,10 @@ __global__ void __launch_bounds__(THREADS, 1) mp_hess_kernel(const __grid_consta
     hm = fmaxf(hm, abs1(h));
   }
   atomicMax(&s_hmax, __float_as_uint(hm));
+  __syncthreads();
+  float sc, un;
+  pow2_scales(__uint_as_float(s_hmax), sc, un);
+  for (int e = tid; e < m * m; e += THREADS) A[e] = scale_f(A[e], sc);
   __syncthreads();
   for (int c = 0; c + 2 < m; ++c) {
     // every warp forms the same reflector (no barrier for it); nr: rows and
@@ -597,7 +605,9 @@ __global__ void __launch_bounds__(kChaseThreads, 1) mp_chase_kernel(const __grid
   C* H = SMEM ? reinterpret_cast<C*>(smem_raw) : D.Hp;
   if (SMEM)
     for (int e = tid; e < offh(m); e += kChaseThreads) H[e] = D.Hp[e];
-  const float hmax = __int_as_float(ctl[D.hmax_slot]);
+  float sc, un;
+  pow2_scales(__int_as_float(ctl[D.hmax_slot]), sc, un);
+  const float hmax = __int_as_float(ctl[D.hmax_slot]) * sc;
   int ihi = m - 1, its = 0, sweeps = 0, step = 0, status = 0;
   if (tid == 0) s_nblk = s_next = s_most = s_bad = 0;
   __syncthreads();
@@ -910,10 +920,16 @@ constexpr bool op_ds(int op) { return op == OP_W || op == OP_G || op == OP_R || 
 struct DsC {
   float rh, rl, ih, il;
 };
+template <bool UNIT>  // UNIT: an entry of orthonormal vectors, of no use below 2^-74
 __device__ __forceinline__ DsC ds_split(double2 v) {
   DsC r;
-  ds::split_flush(v.x, r.rh, r.rl);
-  ds::split_flush(v.y, r.ih, r.il);
+  if constexpr (UNIT) {
+    ds::split_flush(v.x, r.rh, r.rl);
+    ds::split_flush(v.y, r.ih, r.il);
+  } else {
+    ds::split_wide(v.x, r.rh, r.rl);
+    ds::split_wide(v.y, r.ih, r.il);
+  }
   return r;
 }
 
@@ -979,8 +995,8 @@ __global__ void __launch_bounds__(1024) mp_gemm_kernel(const __grid_constant__ M
       const int ka = kb + kk;
       const bool conj_t = OP == OP_G || OP == OP_S;  // a is stored [k][r]: read along r
       const int ar = conj_t ? tx : ty, ak = conj_t ? ty : tx;
-      sa[g][ar][ak] = ds_split(r0 + ar < rows && ka + ak < ke ? lda_d(r0 + ar, ka + ak) : make_double2(0.0, 0.0));
-      sb[g][ty][tx] = ds_split(c0 + tx < cols && ka + ty < ke ? ldb_d(ka + ty, c0 + tx) : make_double2(0.0, 0.0));
+      sa[g][ar][ak] = ds_split<OP != OP_W>(r0 + ar < rows && ka + ak < ke ? lda_d(r0 + ar, ka + ak) : make_double2(0.0, 0.0));
+      sb[g][ty][tx] = ds_split<OP == OP_W || OP == OP_S>(c0 + tx < cols && ka + ty < ke ? ldb_d(ka + ty, c0 + tx) : make_double2(0.0, 0.0));
       __syncthreads();
 #pragma unroll
       for (int q = 0; q < 16; ++q) {

@@ -114,3 +114,21 @@ def test_cut_within_fp32_rounding(ctx, seed):
         assert info[1] == keep
         d = np.abs(np.diag(Tk)[:, None] - th[None, :keep])
         assert d.min(0).max() <= 1e-6  # every one of the keep nearest is there
+
+
+# the grid spacing sets the size of H (~1/h^2): the result scales with it
+@pytest.mark.parametrize("e", [-60, -30, 30, 60])
+@pytest.mark.parametrize("m,keep", [(97, 40), (257, 150)])
+def test_scale_of_the_matrix(ctx, m, keep, e):
+    H = _matrix(m, keep, 2, 7, False)
+    f = 2.0 ** e
+    T, Z, info = ctx.check_restart(H * f, np.zeros((2, m)), keep=keep)
+    assert info[2] == 0, info
+    k = int(info[0])
+    tol = 1e-11 * np.linalg.norm(H)
+    assert np.linalg.norm(H @ Z - Z @ (T / f)) <= tol
+    assert np.abs(Z.conj().T @ Z - np.eye(k)).max() <= 1e-11
+    ev = np.linalg.eigvals(H)
+    ev = ev[np.argsort(np.abs(ev))[:k]]
+    d = np.abs(np.diag(T)[:, None] / f - ev[None, :])
+    assert max(d.min(0).max(), d.min(1).max()) <= 10 * tol
