@@ -23,8 +23,10 @@
 //    the same rows of U at once: half the products, nothing of size N x n stored.
 // FP32 issue bounds all three (4 x 4 complex outputs: 64 FMA per 8 shared loads).
 // Measured on one GB300, 1,000 pairs of 64x64x128, 256 energies: projections
-// 76 ms against 83, adjoint 114 against 167 (all of M, operands converted on
-// the FP64 pipe and loaded between barriers).
+// 73 ms against 83, adjoint 114 against 167 (all of M, operands converted on
+// the FP64 pipe and loaded between barriers).  64 pairs of 32x30x64, 64 energies:
+// projections 0.35 ms against 0.49 (0.44 with Gamma's load left between the
+// barriers), adjoint 0.62 both.
 #include <algorithm>
 #include <cfloat>
 
@@ -103,6 +105,7 @@ __global__ void __launch_bounds__(kThr, 2) proj_f32_kernel(const double2* __rest
   int stage = 0;
   constexpr int kPerP = kKP * kT / kThr;
   double2 pa[kPerP], pc[kPerP];  // the next stage, in flight during this one's products
+  double pg[kPerP];
   const auto fetch = [&](long long r0) {
 #pragma unroll
     for (int u = 0; u < kPerP; ++u) {
@@ -111,6 +114,7 @@ __global__ void __launch_bounds__(kThr, 2) proj_f32_kernel(const double2* __rest
       const double2* Ur = U + r * (long long)ldu;
       pa[u] = r < re && a0 + col < n ? __ldg(Ur + a0 + col) : make_double2(0.0, 0.0);
       pc[u] = r < re && c0 + col < n ? __ldg(Ur + c0 + col) : make_double2(0.0, 0.0);
+      pg[u] = r < re ? __ldg(gam + r) : 0.0;
     }
   };
   fetch(rb);
@@ -118,7 +122,7 @@ __global__ void __launch_bounds__(kThr, 2) proj_f32_kernel(const double2* __rest
 #pragma unroll
     for (int u = 0; u < kPerP; ++u) {
       const int q = threadIdx.x + u * kThr, k = q / kT, col = q % kT;
-      const float g = r0 + k < re ? f1(__ldg(gam + r0 + k)) : 0.f;
+      const float g = f1(pg[u]);
       const float2 v = f2(pa[u]);
       sa[k][col] = make_float2(g * v.x, -g * v.y);
       sc[k][col] = f2(pc[u]);
@@ -228,7 +232,17 @@ __global__ void __launch_bounds__(kThr) gradM_f32_kernel(const float2* __restric
       }
       __syncthreads();
 #pragma unroll
-      for (int ll = 0; ll < kK; ++ll) tile_step(acc, &sr[ll][ty], &sl[ll][tx]);
+      for (int ll = 0; ll < kK; ++ll) {
+        float2 xr[4], xl[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) xr[i] = sr[ll][ty + 16 * i];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) xl[j] = sl[ll][tx + 16 * j];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) fcfma(acc[i][j], xr[i], xl[j]);
+      }
       __syncthreads();
     }
 #pragma unroll
@@ -273,8 +287,11 @@ __global__ void symm_kernel(const float2* __restrict__ M, int n, float2* __restr
 }
 
 // out[r] = 2 Re sum_c U_rc sum_{a <= c} S_ac U_ra for the 64 rows r0 .. r0 + 63 of
-// a block; a stage's operands are loaded during the products of the one before
-__global__ void __launch_bounds__(kThr, 2) rowquad_f32_kernel(const double2* __restrict__ U, int ldu,
+// a block; a stage's operands are loaded during the products of the one before.
+// ONE (a single tile, S = M): nothing to halve, and too few stages to load ahead
+// (64 pairs, 61,440 rows: 79 us, and the launch of symm_kernel less)
+template <bool ONE>
+__global__ void __launch_bounds__(kThr, ONE ? 3 : 2) rowquad_f32_kernel(const double2* __restrict__ U, int ldu,
                                                               const float2* __restrict__ S, int n, long long N,
                                                               double* __restrict__ out) {
   __shared__ float2 su[kK][kT + 1];  // su[a][row] = U[r0 + row][a0 + a]
@@ -308,15 +325,16 @@ __global__ void __launch_bounds__(kThr, 2) rowquad_f32_kernel(const double2* __r
         }
       }
     };
-    fetch(0);
+    if (!ONE) fetch(0);
     for (int a0 = 0; a0 < a1; a0 += kK) {
+      if (ONE) fetch(a0);
 #pragma unroll
       for (int u = 0; u < kPer; ++u) {
         const int q = threadIdx.x + u * kThr;
         su[q % kK][q / kK] = f2(pu[u]);
         sm[q / kT][q % kT] = pm[u];
       }
-      if (a0 + kK < a1) fetch(a0 + kK);
+      if (!ONE && a0 + kK < a1) fetch(a0 + kK);
       __syncthreads();
 #pragma unroll
       for (int aa = 0; aa < kK; ++aa) tile_step(acc, &su[aa][ty], &sm[aa][tx]);
@@ -414,12 +432,18 @@ void launch_grad_f32(const float2* R32, const float2* L32, const double2* eps, i
   gradM_f32_kernel<<<dim3(nt, nt), kThr, 0, s>>>(R32, L32, gt, w, n, nE, M);
   SWI_CHECK_LAUNCH();
   if (launches) ++*launches;
-  const long long nn = (long long)n * n;
-  symm_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(M, n, S);
+  const unsigned rows = (unsigned)((N + kT - 1) / kT);
+  if (nt == 1) {
+    rowquad_f32_kernel<true><<<rows, kThr, 0, s>>>(U, ldu, M, n, N, out);
+  } else {
+    const long long nn = (long long)n * n;
+    symm_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(M, n, S);
+    SWI_CHECK_LAUNCH();
+    if (launches) ++*launches;
+    rowquad_f32_kernel<false><<<rows, kThr, 0, s>>>(U, ldu, S, n, N, out);
+  }
   SWI_CHECK_LAUNCH();
-  rowquad_f32_kernel<<<(unsigned)((N + kT - 1) / kT), kThr, 0, s>>>(U, ldu, S, n, N, out);
-  SWI_CHECK_LAUNCH();
-  if (launches) *launches += 2;
+  if (launches) ++*launches;
 }
 
 }  // namespace swi
