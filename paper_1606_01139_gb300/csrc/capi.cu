@@ -704,6 +704,7 @@ swi_status do_solve(swi_ctx* c, const swi_solve_opts* o, swi_solve_info* info) {
     any_noconv |= (w.nconv < w.nreq);
   }
   win.clear();  // free the Krylov bases before the merge
+  c->pad_ds.release();
   const double t1 = swi::now_seconds();
 
   // ---- Algorithm 2 merge, selection, U^T U = I

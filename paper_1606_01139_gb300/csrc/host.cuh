@@ -80,7 +80,7 @@ struct swi_ctx {
   DevMem V32, G32;  // FP32 copies for the complex64 stencil
   DevMem VG32;      // (V, Gamma) pairs with even row length, for the TMA-staged stencil
   DevMem VGds;      // 8 (V, Gamma) split into floats, for the double-single stencil
-  DevMem pad_ds;    // its padded, split copy of the vectors
+  DevMem pad_ds;    // its padded, split copy of the vectors (kept for repeated swi_apply_ds, given back by a solve)
   bool has_V = false, has_G = false;
   double maxabsV = 0.0, maxG = 0.0;
   std::vector<double> sigma;

@@ -573,6 +573,7 @@ swi_status solve_sv(swi_ctx* c, const swi_solve_opts& opt, swi_solve_info* info)
   Tmp.release();
   Vcur.release();
   Wblk.release();
+  c->pad_ds.release();
   const double t1 = swi::now_seconds();
   int minfo[4];
   merge_pairs(c, c->Uall.as<double2>(), n_all, eps_all, win_of, nwin, eq_rtol, drop_tol, opt.n_keep, minfo);

@@ -196,10 +196,10 @@ __global__ void pack_vg_ds_kernel(const double* __restrict__ V, const double* __
 long long padded(const StencilParams& P) {
   return (long long)(P.nx + 2 * kR) * (P.ny + 2 * kR) * (P.nz + 2 * kR);
 }
-// columns per pass: all of a block of at most 32, fewer when the padded copy
-// would pass 2 GB
+// columns per pass: all of a block of at most 32, fewer (at least one) when the
+// padded copy would pass 2 GB
 int pass_columns(const StencilParams& P, int ncols) {
-  const long long most = std::max<long long>(2, (2LL << 30) / (16 * padded(P)));
+  const long long most = std::max<long long>(1, (2LL << 30) / (16 * padded(P)));
   return (int)std::min<long long>({(long long)ncols, 32, most});
 }
 
