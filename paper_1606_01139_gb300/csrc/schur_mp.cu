@@ -721,7 +721,8 @@ __global__ void __launch_bounds__(kChaseThreads, 1) mp_chase_kernel(const __grid
       int q = 0;
       if (lane == 0) q = atomicAdd(&s_next, 1);
       q = __shfl_sync(0xffffffffu, q, 0);
-      if (q >= nblk || s_bad) break;
+      // one decision for the warp: another warp may set s_bad between two lanes' reads
+      if (q >= nblk || __any_sync(0xffffffffu, s_bad)) break;
       const int l0 = s_small[q].x;
       int top = s_small[q].y, it = 0, total = 0;
       while (top > l0) {
