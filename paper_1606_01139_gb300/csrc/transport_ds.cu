@@ -10,10 +10,11 @@
 // several outputs, real and imaginary parts go through packed FP32x2
 // instructions (half the issue slots; the rest carry loads and splits), and
 // nothing inside the loops touches the FP64 pipe.  Sums run in double-single over
-// at most 1,024 terms and in FP64 beyond.
+// at most 1,024 terms and in FP64 beyond.  Rows of R and L, and S as a whole, are
+// scaled by powers of two before they are split: their sizes follow the absorbers.
 //
 // Measured on one GB300, 400 pairs of the 48x48x96 grid, 128 energies:
-// adjoint 49 ms against 176 (M in native FP64, ~119; U M as an N x n product, then
+// adjoint 52 ms against 176 (M in native FP64, ~119; U M as an N x n product, then
 // a row dot: all of M, and 1.4 GB of scratch).  48 pairs of the 10x10x20 grid, 32
 // energies: 0.10 ms against 2.7.
 #include <algorithm>
@@ -30,6 +31,7 @@ constexpr int kT = 32;     // output tile edge
 constexpr int kK = 16;     // contraction depth of one shared-memory stage
 constexpr int kThr = 256;  // 16 x 16 threads, 2 x 2 outputs each (rows ty + 16 i, columns tx + 16 j)
 constexpr int kFlush = 64;  // stages (1,024 terms) per FP64 flush
+constexpr int kNorm = 8;    // terms between two renormalisations of a running sum
 
 struct V4 {  // complex double-single: heads (re, im), tails (re, im)
   float2 h, l;
@@ -69,9 +71,13 @@ __device__ __forceinline__ void cmac(V4& a, const V4& x, const V4& y) {
   mulv(a, mp(x.h.y), mp(x.l.y), swp(y.h), swp(y.l));
 }
 __device__ __forceinline__ V4 zero4() { return V4{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
+// head + tail as a pair again (TwoSum).  A running sum's tail collects the heads'
+// rounding errors and grows with their number, and its own rounding with it: after
+// k terms ~0.08 k 2^-48 of their root sum of squares (a CPU emulation), with this
+// every 8 terms 0.3 sqrt(k) 2^-48
 __device__ __forceinline__ V4 renorm(const V4& a) {
-  const ds::df r = ds::two_sum(a.h.x, a.l.x), i = ds::two_sum(a.h.y, a.l.y);
-  return V4{make_float2(r.h, i.h), make_float2(r.l, i.l)};
+  const float2 t = add2(a.h, a.l), bb = sub2(t, a.h);
+  return V4{t, add2(sub2(a.h, sub2(t, bb)), sub2(a.l, bb))};
 }
 __device__ __forceinline__ void flush(double2& s, V4& a) {
   s.x += (double)a.h.x + (double)a.l.x;
@@ -165,18 +171,24 @@ __global__ void __launch_bounds__(kThr, 2)
         sl[ll][row] = v;
       }
       __syncthreads();
+      for (int lb = 0; lb < kK; lb += kNorm) {
 #pragma unroll 4
-      for (int ll = 0; ll < kK; ++ll) {
-        V4 xr[2], xl[2];
+        for (int ll = lb; ll < lb + kNorm; ++ll) {
+          V4 xr[2], xl[2];
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          xr[i] = ld(sr[ll][ty + 16 * i]);
-          xl[i] = ld(sl[ll][tx + 16 * i]);
+          for (int i = 0; i < 2; ++i) {
+            xr[i] = ld(sr[ll][ty + 16 * i]);
+            xl[i] = ld(sl[ll][tx + 16 * i]);
+          }
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) cmac(acc[i][j], xr[i], xl[j]);
         }
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
-          for (int j = 0; j < 2; ++j) cmac(acc[i][j], xr[i], xl[j]);
+          for (int j = 0; j < 2; ++j) acc[i][j] = renorm(acc[i][j]);
       }
       __syncthreads();
       if (++stage == kFlush) {
@@ -276,18 +288,24 @@ __global__ void __launch_bounds__(kThr, 2)
         }
       }
       __syncthreads();
+      for (int ab = 0; ab < kK; ab += kNorm) {
 #pragma unroll 4
-      for (int aa = 0; aa < kK; ++aa) {
-        V4 xu[2], xm[2];
+        for (int aa = ab; aa < ab + kNorm; ++aa) {
+          V4 xu[2], xm[2];
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          xu[i] = ld(su[aa][ty + 16 * i]);
-          xm[i] = ld(sm[aa][tx + 16 * i]);
+          for (int i = 0; i < 2; ++i) {
+            xu[i] = ld(su[aa][ty + 16 * i]);
+            xm[i] = ld(sm[aa][tx + 16 * i]);
+          }
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) cmac(acc[i][j], xu[i], xm[j]);
         }
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
-          for (int j = 0; j < 2; ++j) cmac(acc[i][j], xu[i], xm[j]);
+          for (int j = 0; j < 2; ++j) acc[i][j] = renorm(acc[i][j]);
       }
       __syncthreads();
     }
