@@ -53,8 +53,8 @@ WORKLOAD = "wire_48x48x96"
 METRIC = "converged eigenpairs/s at rel residual 1e-8"
 UNIT = "eigenpairs/s"
 REL_TOL = 1e-8
-# Per-window budget of operator applications (vectors), sized so that one step
-# takes about two minutes.  Windows that have not converged within it deliver
+# Per-window budget of operator applications (vectors); one step takes about a
+# minute.  Windows that have not converged within it deliver
 # what they have; only pairs whose explicit FP64 residual is <= REL_TOL are
 # counted.  (The upper windows of this spectrum need 150,000 and more.)
 MATVEC_BUDGET = 20000

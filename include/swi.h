@@ -95,8 +95,12 @@ typedef struct {
                            m_j - b) */
   int arith;            /* arithmetic of the Krylov loop and T(E):
                            0 or SWI_ARITH_DS (default) -- stencil, Cholesky-QR,
-                           projected Schur step and T(E) projections in
-                           double-single on the FP32 pipes; for b <= 2 the
+                           T(E) projections and the adjoint in double-single on
+                           the FP32 pipes; projected Schur step from an FP32
+                           Schur form, the kept subspace and its triangle
+                           corrected to double-single (residual at most 1e-13
+                           of the largest entry), by the double-single step of
+                           full order where that fails; for b <= 2 the
                            Gram-Schmidt passes as described with the kernels
                            (FP32 first Gram and second update, double-single
                            accurate pass), for b >= 3 Gram-Schmidt products and
@@ -260,8 +264,12 @@ swi_status swi_apply(swi_ctx* ctx, int nvec, const double* sigma, const void* X,
 
 /* swi_apply in double-single arithmetic (the operator of the double-single
  * Krylov loop): same arguments, complex128 in and out; every input value is
- * split into two floats and each of the 37 terms is an exact FMA product
- * summed with TwoSum, ~2^-48 relative per term.  Errors as swi_apply. */
+ * split into two floats; per distance the six neighbours are summed (TwoSum)
+ * and multiplied by the weight once (FMA, the tail kept), ~2^-47 relative per
+ * term.  The range is that of a float: entries beyond it count as infinite,
+ * infinities and NaN reach the outputs that they reach in 64 bits.  The context
+ * keeps a padded copy of X between calls (at most 2 GB, or one column).
+ * Errors as swi_apply. */
 swi_status swi_apply_ds(swi_ctx* ctx, int nvec, const double* sigma, const void* X, void* Y,
                         int on_device);
 

@@ -3,10 +3,12 @@
 // The host plans and sequences; every O(N) step runs in this library's
 // kernels on the context's stream.  One solve batches all windows (the
 // paper's independent partitions, Section 2.1) into shared launches: the
-// stencil applies (A - sigma_j) to the new block of every active window in one
-// launch, the orthogonalisation and Cholesky-QR of all windows go out as
-// batched launches, and windows that reach their maximum basis restart
-// together.  The host reads back only a few status words per restart.
+// orthogonalisation and Cholesky-QR of all windows go out as batched launches,
+// the operator as one call for all windows of 1 or 2 vectors (wide blocks window
+// by window in double-single: 59 us a step for four windows of 16 vectors on
+// 24x22x48, 181 us as one launch of the form before the padded copy), and a window
+// that reaches its maximum basis restarts on a stream of its own.  The host reads
+// back only a few status words per restart.
 #include <algorithm>
 #include <cfloat>
 #include <cmath>

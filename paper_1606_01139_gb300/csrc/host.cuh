@@ -1,6 +1,6 @@
 // Host-side state of a solver context, shared by the translation units that
-// drive the solves (capi.cu: the C ABI and the double-single solver;
-// solve_mixed.cu: the complex64 single-vector solver).
+// drive the solves (capi.cu: the C ABI and the wide-block solver; solve_sv.cu:
+// the windows of 1 or 2 vectors, double-single or complex64).
 #pragma once
 
 #include <algorithm>

@@ -452,7 +452,7 @@ swi_status solve_sv(swi_ctx* c, const swi_solve_opts& opt, swi_solve_info* info)
       if (q == cudaErrorNotReady) continue;
       SWI_CUDA_TRY(q);
       in_schur[j] = 0;
-      finish_restart(j);  // may start the FP64 retry (in_schur set again)
+      finish_restart(j);  // may start the next form (in_schur set again)
     }
     std::vector<Win*> act;
     int pending = -1;
