@@ -110,7 +110,7 @@ swi::StencilParams stencil_params(const swi_ctx* c) {
   for (int m = 0; m < 7; ++m) P.cm[m] = -kFD[m] / (2.0 * c->h * c->h);
   P.V = c->V.as<double>();
   P.G = c->G.as<double>();
-  P.VGds = c->VGds.as<float4>();
+  P.VGds = c->vgds();
   return P;
 }
 
@@ -1124,11 +1124,9 @@ swi_status swi_create(swi_ctx** out, int nx, int ny, int nz, double h, int bc, i
 // the packed (V, Gamma) arrays of the TMA-staged complex64 and the double-single stencils, once both are set
 static void refresh_vg(swi_ctx* c) {
   if (!c->has_V || !c->has_G) return;
-  const size_t nxp = (size_t)(c->nx + (c->nx & 1));
-  c->VG32.ensure(sizeof(float2) * nxp * c->ny * c->nz);
-  c->VGds.ensure(sizeof(float4) * (size_t)c->N);
-  swi::launch_pack_vg_ds(c->V.as<double>(), c->G.as<double>(), c->N, c->VGds.as<float4>(), c->stream);
-  swi::launch_pack_vg(c->V32.as<float>(), c->G32.as<float>(), c->nx, c->ny, c->nz, c->VG32.as<float2>(), c->stream);
+  c->VGpack.ensure(c->vg32_bytes() + sizeof(float4) * (size_t)c->N);
+  swi::launch_pack_vg_ds(c->V.as<double>(), c->G.as<double>(), c->N, c->vgds(), c->stream);
+  swi::launch_pack_vg(c->V32.as<float>(), c->G32.as<float>(), c->nx, c->ny, c->nz, c->vg32(), c->stream);
   sync(c->stream);
 }
 
@@ -1326,7 +1324,7 @@ swi_status swi_apply_c64(swi_ctx* c, int nvec, const float* sigma, const void* X
     for (int m = 0; m < 7; ++m) P.cm[m] = (float)(-kFD[m] / (2.0 * c->h * c->h));
     P.V = c->V32.as<float>();
     P.G = c->G32.as<float>();
-    P.VG = c->VG32.as<float2>();
+    P.VG = c->vg32();
     const double Nn = (double)c->N;
     if (on_device) {
       ProfScope ps(c, SWI_K_STENCIL, kStencilFlops * Nn * nvec, (16.0 * nvec + 8.0) * Nn);

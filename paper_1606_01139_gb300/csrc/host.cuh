@@ -78,8 +78,14 @@ struct swi_ctx {
   int bc = SWI_BC_ODD, precision = SWI_PREC_F64;
   DevMem V, G, gL, gR;
   DevMem V32, G32;  // FP32 copies for the complex64 stencil
-  DevMem VG32;      // (V, Gamma) pairs with even row length, for the TMA-staged stencil
-  DevMem VGds;      // 8 (V, Gamma) split into floats, for the double-single stencil
+  // one allocation: (V, Gamma) pairs with even row length, for the TMA-staged
+  // stencil, then 8 (V, Gamma) split into floats, for the double-single stencil
+  DevMem VGpack;
+  float2* vg32() const { return VGpack.as<float2>(); }
+  float4* vgds() const {
+    return VGpack.p ? reinterpret_cast<float4*>(VGpack.as<char>() + vg32_bytes()) : nullptr;
+  }
+  size_t vg32_bytes() const { return (sizeof(float2) * (size_t)(nx + (nx & 1)) * ny * nz + 255) & ~size_t(255); }
   DevMem pad_ds;    // its padded, split copy of the vectors (kept for repeated swi_apply_ds, given back by a solve)
   bool has_V = false, has_G = false;
   double maxabsV = 0.0, maxG = 0.0;

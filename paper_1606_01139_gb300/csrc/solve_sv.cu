@@ -114,7 +114,7 @@ swi::StencilC64Params stencil_c64_params(const swi_ctx* c) {
   for (int m = 0; m < 7; ++m) P.cm[m] = (float)(-kFD[m] / (2.0 * c->h * c->h));
   P.V = c->V32.as<float>();
   P.G = c->G32.as<float>();
-  P.VG = c->VG32.as<float2>();
+  P.VG = c->vg32();
   return P;
 }
 
